@@ -90,8 +90,23 @@ extern "C" void paam_destroy(paam_ctx *c)
 }
 
 // ---------------------------------------------------------------------------
-// validation: one thread per system; the first failing code wins
+// validation: G = 4 lanes per system, over its chains, then its callbacks, then
+// its segments; the first failing code wins.  What bounds it is the latency of its
+// dependent loads (system -> chain -> callback -> segment) and the instructions
+// around them, so a warp holds eight systems, whose set-up, votes and reductions
+// share each instruction, and neighbouring lanes read neighbouring elements.
+// Nothing is summed per chain: the sums of a system stand for its chains' in the
+// range test, which is taken in single precision with a factor of two in hand, and
+// in the batch maxima; a batch with a system that is not clearly inside the limits
+// takes range_kernel too, whose sums are per chain and whose last word is in double
+// precision (16 cycles per warp instruction on this chip).  A thread per system,
+// sums in double precision: 740 us for 200,000 systems of 8-16 chains, 7,290 us for
+// 1,000,000 of 2-64, 28 us for 1,000 of 4; now 140, 870 and 17 us (16 lanes per
+// system: 202 and 1,002 us; 8 lanes: 158 and 940; six or eight blocks per SM spill:
+// 154 us).  The one read of every table would take 55 us for the 200,000.
 // ---------------------------------------------------------------------------
+
+constexpr int G = 4, kValThreads = 256, kValBlocks = 5;
 
 struct ValidateArgs {
     BatchDev b;
@@ -102,163 +117,300 @@ struct ValidateArgs {
     ValidateRange r;
     int sentinels;
     const int32_t *acc;
-    int32_t *err; // [0] code, [1] first bad system (min), [2] max chains, [3] max executors
+    int32_t *err; // [0] code, [1] 0: the test per chain is needed too, [2] max chains, [3] max executors
     unsigned long long *stats; // ST_* maxima
 };
 
-__device__ __forceinline__ void fail(int32_t *err, int32_t code, int64_t sys)
+__device__ __forceinline__ void fail(int32_t *err, int32_t code) { atomicCAS(&err[0], 0, code); }
+
+// The range and iteration tests of one system whose tables passed every other
+// check, in double precision (exact up to 2^53) and int64.
+__device__ __noinline__ bool range_exact(const BatchDev &b, int64_t c0, int64_t c1)
 {
-    atomicCAS(&err[0], 0, code);
-    atomicMin(&err[1], (int32_t)(sys < 0x7fffffff ? sys : 0x7fffffff));
+    const double OV = (double)PAAM_MAX_OVERHEAD;
+    double Dmax = 0.0, Tmin = 1e300, Cmax = 0.0, Base = 0.0, Emax = 0.0, Mmax = 0.0, dseg_max = 0.0;
+    for (int64_t c = c0; c < c1; ++c) {
+        const int64_t cb0 = b.chain_cb_off[c], cb1 = b.chain_cb_off[c + 1];
+        double Ec = 0.0, Sc = 0.0;
+        for (int64_t cb = cb0; cb < cb1; ++cb) {
+            Ec += (double)b.E[cb];
+            Emax = fmax(Emax, (double)b.E[cb]);
+        }
+        const int64_t q0 = b.cb_seg_off[cb0], q1 = b.cb_seg_off[cb1];
+        for (int64_t q = q0; q < q1; ++q) {
+            const double as = (double)b.A[q] + 2.0 * OV;
+            Sc += as;
+            Mmax = fmax(Mmax, as);
+        }
+        const double dc = (double)(q1 - q0), D = (double)b.D[c];
+        Dmax = fmax(Dmax, D);
+        Tmin = fmin(Tmin, (double)b.T[c]);
+        Cmax = fmax(Cmax, Ec + fmax(D, dc * OV) + Sc);
+        Base = fmax(Base, Ec + Sc + dc * OV);
+        dseg_max = fmax(dseg_max, dc);
+    }
+    // the largest value an iterate can take: interference over n chains with at most
+    // ceil(Dmax/Tmin)+1 arrivals each, plus blocking and the chain's own demand
+    const double m = ceil(Dmax / Tmin) + 1.0;
+    const double bound = (double)(c1 - c0) * m * Cmax + Base + Emax + dseg_max * Mmax + Dmax;
+    if (!(bound < 2.305843009213694e18)) return false; /* 2^61: margin under 2^62 */
+    // iteration bound: after its first step a recurrence rises only when an
+    // arrival count ceil(t / T_h) + 1 (Lemma 1) has grown, at most
+    // ceil(Dmax / T_h) times per chain h while t <= Dmax
+    const uint64_t Dm = (uint64_t)Dmax; // exact: at most 2^40
+    uint64_t iters = 2;
+    for (int64_t c = c0; c < c1 && iters <= (uint64_t)PAAM_MAX_ITER; ++c) {
+        const uint64_t T = (uint64_t)b.T[c];
+        iters += (Dm + T - 1) / T;
+    }
+    return iters <= (uint64_t)PAAM_MAX_ITER;
 }
 
-__global__ void validate_kernel(ValidateArgs a)
+// A batch maximum that is seldom raised.
+__device__ __forceinline__ void raise_max(unsigned long long *at, unsigned long long v)
+{
+    if (v > *(volatile unsigned long long *)at) atomicMax(at, v);
+}
+
+// The range test of a system that passed every other check, and its chains' part
+// in the batch maxima, from 64-bit sums per chain, one chain per lane; what is
+// not clear in single precision is decided exactly.
+__device__ __forceinline__ void range_per_chain(const ValidateArgs &a, int64_t s, int lane, unsigned gm)
 {
     const BatchDev &b = a.b;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    unsigned long long lmax[ST_COUNT] = {};
-    int32_t nmax = 0, xmax = 0;
-    for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < b.n_sys; s += stride) {
-        if (s == 0 && a.sentinels) { // global sentinels
-            if (b.sys_chain_off[0] != 0 || b.sys_exec_off[0] != 0 || b.chain_cb_off[0] != 0 ||
-                b.cb_seg_off[0] != 0 || b.sys_chain_off[b.n_sys] != a.n_chain ||
-                b.sys_exec_off[b.n_sys] != a.n_exec || b.chain_cb_off[a.n_chain] != a.n_cb ||
-                b.cb_seg_off[a.n_cb] != a.n_seg) {
-                fail(a.err, PAAM_E_INVAL, s);
-                continue;
-            }
+    const int64_t c0 = b.sys_chain_off[s], c1 = b.sys_chain_off[s + 1];
+    float Cmax = 0.0f, Mmax = 0.0f, dsegs = 0.0f, Dmax = 0.0f, Tmin = 3e38f;
+    for (int64_t c = c0 + lane; c < c1; c += G) {
+        const int64_t cb0 = b.chain_cb_off[c], cb1 = b.chain_cb_off[c + 1];
+        unsigned long long E = 0, S = 0, M = 0;
+        for (int64_t cb = cb0; cb < cb1; ++cb) E += (unsigned long long)b.E[cb];
+        const int64_t q0 = b.cb_seg_off[cb0], q1 = b.cb_seg_off[cb1];
+        for (int64_t q = q0; q < q1; ++q) {
+            const unsigned long long v = (unsigned long long)b.A[q];
+            S += v;
+            M = max(M, v);
         }
+        raise_max(&a.stats[ST_TMAX], (unsigned long long)b.T[c]);
+        raise_max(&a.stats[ST_DMAX], (unsigned long long)b.D[c]);
+        raise_max(&a.stats[ST_ECMAX], E);
+        raise_max(&a.stats[ST_SCMAX], S);
+        raise_max(&a.stats[ST_DELTAMAX], (unsigned long long)(q1 - q0));
+        const float dc = (float)(q1 - q0), D = (float)b.D[c];
+        Cmax = fmaxf(Cmax, (float)E + fmaxf(D, dc * 0x1p32f) + (float)S + dc * 0x1p33f);
+        if (cb1 - cb0 >= (1 << 20)) Cmax = 0x1p100f; // their sum may have wrapped: decided exactly
+        if (q1 > q0) Mmax = fmaxf(Mmax, (float)M + 0x1p33f); // a wrapped sum of A has dc Mmax >= 2^64
+        dsegs = fmaxf(dsegs, dc);
+        Dmax = fmaxf(Dmax, D);
+        Tmin = fminf(Tmin, (float)b.T[c]);
+    }
+    Cmax = __uint_as_float(__reduce_max_sync(gm, __float_as_uint(Cmax))); // bits order as non-negative floats do
+    Mmax = __uint_as_float(__reduce_max_sync(gm, __float_as_uint(Mmax)));
+    dsegs = __uint_as_float(__reduce_max_sync(gm, __float_as_uint(dsegs)));
+    Dmax = __uint_as_float(__reduce_max_sync(gm, __float_as_uint(Dmax)));
+    Tmin = __uint_as_float(__reduce_min_sync(gm, __float_as_uint(Tmin)));
+    const float ratio = Dmax / Tmin, n = (float)(c1 - c0);
+    const bool clear = c1 == c0 || ((n * (ratio + 2.0f) + 3.0f) * Cmax + dsegs * Mmax < 0x1p60f &&
+                                    n * (ratio + 1.0f) + 2.0f < 0.5f * (float)PAAM_MAX_ITER);
+    if (!clear && lane == 0 && !range_exact(b, c0, c1)) fail(a.err, PAAM_E_RANGE);
+    __syncwarp(gm);
+}
+
+// Every system of a batch that validate_kernel found valid but could not place
+// clearly inside the limits (rare: periods of seconds, thousands of segments,
+// magnitudes near the limits); a launch of its own, so that the pass that every
+// batch takes keeps its registers.
+__global__ void __launch_bounds__(kValThreads) range_kernel(const __grid_constant__ ValidateArgs a)
+{
+    const int lane = threadIdx.x % G;
+    const unsigned gm = ((1u << G) - 1u) << (threadIdx.x & 31u & ~(unsigned)(G - 1));
+    const int64_t stride = (int64_t)gridDim.x * (kValThreads / G);
+    for (int64_t s = (int64_t)blockIdx.x * (kValThreads / G) + threadIdx.x / G; s < a.b.n_sys; s += stride)
+        range_per_chain(a, s, lane, gm);
+}
+
+// Per lane sums of E and A are taken up to kLaneCap (a group's sum fits 32 bits),
+// and a system's sums below kSumCap stand for its chains' in the batch maxima.
+constexpr uint32_t kLaneCap = (1u << 28) - 1, kSumCap = 1u << 29;
+
+__global__ void __launch_bounds__(kValThreads, kValBlocks) validate_kernel(const __grid_constant__ ValidateArgs a)
+{
+    __shared__ unsigned long long part[8][ST_COUNT + 2];
+    const BatchDev &b = a.b;
+    const int lane = threadIdx.x % G;
+    const unsigned gm = ((1u << G) - 1u) << (threadIdx.x & 31u & ~(unsigned)(G - 1));
+    const int64_t stride = (int64_t)gridDim.x * (kValThreads / G);
+    uint32_t tmax = 0, dmax = 0, ecmax = 0, scmax = 0, dlmax = 0, accmax = 0;
+    int32_t nmax = 0, xmax = 0;
+    bool again = false; // one of the group's systems needs the test per chain
+    for (int64_t s = (int64_t)blockIdx.x * (kValThreads / G) + threadIdx.x / G; s < b.n_sys; s += stride) {
         const int64_t c0 = b.sys_chain_off[s], c1 = b.sys_chain_off[s + 1];
         const int64_t x0 = b.sys_exec_off[s], x1 = b.sys_exec_off[s + 1];
-        if (c0 < a.r.chain_lo || c1 < c0 || c1 > a.r.chain_hi || x0 < a.r.exec_lo || x1 < x0 ||
-            x1 > a.r.exec_hi) {
-            fail(a.err, PAAM_E_INVAL, s);
-            continue;
-        }
-        const int64_t n = c1 - c0, nx = x1 - x0;
-        if (n > PAAM_MAX_CHAINS || (n > 0 && nx == 0)) {
-            fail(a.err, PAAM_E_INVAL, s);
-            continue;
-        }
-        nmax = (int32_t)n > nmax ? (int32_t)n : nmax;
-        const int32_t nx32 = (int32_t)(nx < 0x7fffffff ? nx : 0x7fffffff);
-        xmax = nx32 > xmax ? nx32 : xmax;
-        // executors
-        bool bad = false;
-        for (int64_t x = x0; x < x1 && !bad; ++x) {
-            if (b.exec_core[x] < 0) bad = true;
-            if (b.exec_prio)
-                for (int64_t y = x0; y < x && !bad; ++y)
-                    if (b.exec_core[y] == b.exec_core[x] && b.exec_prio[y] == b.exec_prio[x]) bad = true;
-        }
+        const int64_t nx = x1 - x0;
+        // every lane of the group sees the same offsets and takes the same path
+        bool bad = c0 < a.r.chain_lo || c1 < c0 || c1 > a.r.chain_hi || x0 < a.r.exec_lo || x1 < x0 ||
+                   x1 > a.r.exec_hi || c1 - c0 > PAAM_MAX_CHAINS || (c1 > c0 && nx == 0);
+        if (s == 0 && a.sentinels) // global sentinels
+            bad |= b.sys_chain_off[0] != 0 || b.sys_exec_off[0] != 0 || b.chain_cb_off[0] != 0 ||
+                   b.cb_seg_off[0] != 0 || b.sys_chain_off[b.n_sys] != a.n_chain ||
+                   b.sys_exec_off[b.n_sys] != a.n_exec || b.chain_cb_off[a.n_chain] != a.n_cb ||
+                   b.cb_seg_off[a.n_cb] != a.n_seg;
         if (bad) {
-            fail(a.err, PAAM_E_INVAL, s);
+            if (lane == 0) fail(a.err, PAAM_E_INVAL);
             continue;
         }
-        // chains, callbacks, segments; magnitudes for the range check
-        double Dmax = 0.0, Tmin = 1e300, Cmax = 0.0, Base = 0.0, Emax_sys = 0.0, Mmax_sys = 0.0;
-        const double OV = (double)PAAM_MAX_OVERHEAD;
-        for (int64_t c = c0; c < c1 && !bad; ++c) {
-            const int64_t T = b.T[c], D = b.D[c];
-            if (T <= 0 || T > PAAM_MAX_TIME || D <= 0 || D > T || b.spin[c] > 1 || b.exec[c] < 0 ||
-                b.exec[c] >= nx) {
-                bad = true;
-                break;
-            }
-            for (int64_t k = c0; k < c; ++k)
-                if (b.prio[k] == b.prio[c]) bad = true;
-            const int64_t b0 = b.chain_cb_off[c], b1 = b.chain_cb_off[c + 1];
-            if (b0 < a.r.cb_lo || b1 < b0 || b1 > a.r.cb_hi) {
-                bad = true;
-                break;
-            }
-            double Ec = 0.0, Sc = 0.0, dc = 0.0;
-            unsigned long long Ei = 0, Si = 0, di = 0;
-            for (int64_t cb = b0; cb < b1 && !bad; ++cb) {
-                const int64_t e = b.E[cb];
-                const int64_t q0 = b.cb_seg_off[cb], q1 = b.cb_seg_off[cb + 1];
-                if (e < 0 || e > PAAM_MAX_TIME || q0 < a.r.seg_lo || q1 < q0 || q1 > a.r.seg_hi) {
-                    bad = true;
-                    break;
-                }
-                Ec += (double)e;
-                Ei += (unsigned long long)e;
-                if ((double)e > Emax_sys) Emax_sys = (double)e;
-                for (int64_t q = q0; q < q1; ++q) {
-                    const int64_t av = b.A[q];
-                    if (av < 0 || av > PAAM_MAX_TIME) {
-                        bad = true;
-                        break;
-                    }
-                    if (a.acc) { // one server per accelerator (R1), up to PAAM_MAX_ACC of them
-                        const int32_t u = a.acc[q];
-                        if (u < 0 || u >= PAAM_MAX_ACC) {
-                            bad = true;
-                            break;
-                        }
-                        lmax[ST_ACCMAX] = max(lmax[ST_ACCMAX], (unsigned long long)u);
-                    }
-                    const double as = (double)av + 2.0 * OV;
-                    Sc += as;
-                    dc += 1.0;
-                    Si += (unsigned long long)av;
-                    di += 1;
-                    if (as > Mmax_sys) Mmax_sys = as;
-                }
-            }
-            if ((double)D > Dmax) Dmax = (double)D;
-            if ((double)T < Tmin) Tmin = (double)T;
-            lmax[ST_TMAX] = max(lmax[ST_TMAX], (unsigned long long)T);
-            lmax[ST_DMAX] = max(lmax[ST_DMAX], (unsigned long long)D);
-            lmax[ST_ECMAX] = max(lmax[ST_ECMAX], Ei);
-            lmax[ST_SCMAX] = max(lmax[ST_SCMAX], Si);
-            lmax[ST_DELTAMAX] = max(lmax[ST_DELTAMAX], di);
-            const double spin_or_d = (double)D > dc * OV ? (double)D : dc * OV;
-            const double C = Ec + spin_or_d + Sc;
-            if (C > Cmax) Cmax = C;
-            const double base = Ec + Sc + dc * OV;
-            if (base > Base) Base = base;
+        const int n = (int)(c1 - c0);
+        nmax = max(nmax, n);
+        xmax = max(xmax, (int32_t)(nx < 0x7fffffff ? nx : 0x7fffffff));
+        // the system's callbacks and, once their offsets are known to be in range, segments
+        const int64_t b0 = b.chain_cb_off[c0], b1 = b.chain_cb_off[c1];
+        bad = n > 0 && (b0 < a.r.cb_lo || b1 > a.r.cb_hi);
+        // chains (times of 2^32 ns and more: the test per chain)
+        uint32_t thi = 0, tlo = 0, dlo = 0, tmin = 0xffffffffu;
+        uint32_t plo = 0, phi = 0; // priorities below 64 (usual: a permutation of 0..n-1) as a set
+        bool pout = false;
+#pragma unroll 2
+        for (int i = lane; i < n; i += G) {
+            const int64_t T = b.T[c0 + i], D = b.D[c0 + i];
+            const int32_t ex = b.exec[c0 + i], pr = b.prio[c0 + i];
+            pout |= (uint32_t)pr >= 64u;
+            if (pr & 32) phi |= 1u << (pr & 31);
+            else plo |= 1u << (pr & 31);
+            bad |= T <= 0 || T > PAAM_MAX_TIME || D <= 0 || D > T || b.spin[c0 + i] > 1 || ex < 0 || ex >= nx ||
+                   b.chain_cb_off[c0 + i + 1] < b.chain_cb_off[c0 + i];
+            thi |= (uint32_t)((uint64_t)T >> 32);
+            tlo = max(tlo, (uint32_t)T);
+            dlo = max(dlo, (uint32_t)D);
+            tmin = min(tmin, (uint32_t)T);
         }
-        if (bad) {
-            fail(a.err, PAAM_E_INVAL, s);
+        // executors: cores, distinct priorities on one core
+        for (int64_t x = x0 + lane; x < x1; x += G) {
+            const int32_t core = b.exec_core[x];
+            bad |= core < 0;
+            if (b.exec_prio) {
+                const int32_t pr = b.exec_prio[x];
+                for (int64_t y = x0; y < x; ++y) bad |= b.exec_prio[y] == pr && b.exec_core[y] == core;
+            }
+        }
+        // distinct chain priorities: the set has n members, or one comparison per pair
+        plo = __reduce_or_sync(gm, plo);
+        phi = __reduce_or_sync(gm, phi);
+        if (__any_sync(gm, pout)) {
+            const int32_t *P = b.prio + c0;
+            for (int i = lane; i < n; i += G)
+                for (int k = 0; k < i; ++k) bad |= P[k] == P[i];
+        } else {
+            bad |= __popc(plo) + __popc(phi) != n;
+        }
+        if (__any_sync(gm, bad)) {
+            if (lane == 0) fail(a.err, PAAM_E_INVAL);
             continue;
         }
-        if (n > 0) {
-            // the largest value an iterate can take: interference over n chains with at most
-            // ceil(Dmax/Tmin)+1 arrivals each, plus blocking and the chain's own demand
-            double dseg_max = 0.0;
-            for (int64_t c = c0; c < c1; ++c)
-                dseg_max = fmax(dseg_max, (double)(b.cb_seg_off[b.chain_cb_off[c + 1]] -
-                                                   b.cb_seg_off[b.chain_cb_off[c]]));
-            const double m = ceil(Dmax / Tmin) + 1.0;
-            const double bound = (double)n * m * Cmax + Base + Emax_sys + dseg_max * Mmax_sys + Dmax;
-            if (!(bound < 2.305843009213694e18)) /* 2^61: margin under 2^62 */
-                fail(a.err, PAAM_E_RANGE, s);
-            // iteration bound: after its first step a recurrence rises only when an
-            // arrival count ceil(t / T_h) + 1 (Lemma 1) has grown, at most
-            // ceil(Dmax / T_h) times per chain h while t <= Dmax
-            const uint64_t Dm = (uint64_t)Dmax; // exact: below 2^40
-            uint64_t iters = 2;
-            for (int64_t c = c0; c < c1 && iters <= (uint64_t)PAAM_MAX_ITER; ++c) {
-                const uint64_t T = (uint64_t)b.T[c];
-                iters += (Dm + T - 1) / T;
+        if (n == 0) continue;
+        int64_t q0 = 0, q1 = 0;
+        if (b1 > b0) {
+            q0 = b.cb_seg_off[b0];
+            q1 = b.cb_seg_off[b1];
+            bad = q0 < a.r.seg_lo || q1 > a.r.seg_hi;
+        }
+        // callbacks: E in range (its high words first), segment offsets that do not fall
+        uint64_t es = 0, as = 0;
+        uint32_t ehi = 0, ahi = 0, amax = 0;
+        {
+            const int64_t *Ep = b.E + b0 + lane, *Qp = b.cb_seg_off + b0 + lane;
+            const int64_t m = b1 - b0;
+#pragma unroll 4
+            for (int64_t i = lane; i < m; i += G, Ep += G, Qp += G) {
+                const uint64_t e = (uint64_t)*Ep;
+                bad |= Qp[1] < Qp[0];
+                ehi |= (uint32_t)(e >> 32);
+                es += e;
             }
-            if (iters > (uint64_t)PAAM_MAX_ITER) fail(a.err, PAAM_E_RANGE, s);
+            if (ehi >> 8) // some value at or above 2^40, or negative
+                for (int64_t i = lane; i < m; i += G) bad |= (uint64_t)b.E[b0 + i] > (uint64_t)PAAM_MAX_TIME;
+        }
+        if (__any_sync(gm, bad)) {
+            if (lane == 0) fail(a.err, PAAM_E_INVAL);
+            continue;
+        }
+        // segments: the offsets rise from q0 to q1 inside the range
+        const int64_t dl = q1 - q0;
+        {
+            const int64_t *Ap = b.A + q0 + lane;
+#pragma unroll 4
+            for (int64_t i = lane; i < dl; i += G, Ap += G) {
+                const uint64_t v = (uint64_t)*Ap;
+                ahi |= (uint32_t)(v >> 32);
+                amax = max(amax, (uint32_t)v);
+                as += v;
+            }
+            if (ahi >> 8)
+                for (int64_t i = lane; i < dl; i += G) bad |= (uint64_t)b.A[q0 + i] > (uint64_t)PAAM_MAX_TIME;
+        }
+        if (a.acc) { // one server per accelerator (R1), up to PAAM_MAX_ACC of them
+            uint32_t u = 0;
+#pragma unroll 4
+            for (int64_t i = lane; i < dl; i += G) u = max(u, (uint32_t)a.acc[q0 + i]);
+            bad |= u >= PAAM_MAX_ACC;
+            accmax = max(accmax, u);
+        }
+        if (__any_sync(gm, bad)) {
+            if (lane == 0) fail(a.err, PAAM_E_INVAL);
+            continue;
+        }
+        // Range: with the system's sums E and S over all its chains and its segment count
+        // dl, no chain's demand exceeds C = E + max(Dmax, dl OV) + S + 2 dl OV, and the
+        // largest iterate n (ceil(Dmax / Tmin) + 1) C + 3 C + dl (largest A + 2 OV); a
+        // recurrence takes at most n (Dmax / Tmin + 1) + 2 evaluations.  The floats are
+        // within 2^-20 of their values, so a test at half of each limit is safe; a
+        // system that does not pass it is decided exactly.
+        const float Dm = (float)__reduce_max_sync(gm, dlo), Tm = (float)__reduce_min_sync(gm, tmin);
+        const uint32_t E = __reduce_add_sync(gm, es < kLaneCap ? (uint32_t)es : kLaneCap);
+        const uint32_t S = __reduce_add_sync(gm, as < kLaneCap ? (uint32_t)as : kLaneCap);
+        const float M = (float)__reduce_max_sync(gm, amax) + 0x1p33f;
+        const bool large = __any_sync(gm, es >= kLaneCap || as >= kLaneCap || thi != 0) || E >= kSumCap ||
+                           S >= kSumCap || dl >= (1 << 20);
+        const float ratio = Dm / Tm, nf = (float)n, d32 = (float)dl * 0x1p32f;
+        const float C = (float)E + fmaxf(Dm, d32) + (float)S + 2.0f * d32;
+        if (large || !((nf * (ratio + 2.0f) + 3.0f) * C + (float)dl * M < 0x1p60f &&
+                       nf * (ratio + 1.0f) + 2.0f < 0.5f * (float)PAAM_MAX_ITER)) {
+            again = true;
+            continue;
+        }
+        tmax = max(tmax, tlo);
+        dmax = max(dmax, dlo);
+        ecmax = max(ecmax, E);
+        scmax = max(scmax, S);
+        dlmax = max(dlmax, (uint32_t)dl);
+    }
+    if (again && lane == 0) a.err[1] = 0;
+    static_assert(PAAM_MAX_OVERHEAD == 1ll << 32 && PAAM_MAX_TIME == 1ll << 40, "the limits spelt out above");
+    // the block's maxima, one atomic each, and none where the maximum is there already
+    __syncwarp();
+    unsigned long long v[ST_COUNT + 2];
+    v[ST_TMAX] = tmax;
+    v[ST_DMAX] = dmax;
+    v[ST_ECMAX] = ecmax;
+    v[ST_SCMAX] = scmax;
+    v[ST_DELTAMAX] = dlmax;
+    v[ST_ACCMAX] = accmax;
+    v[ST_COUNT] = (unsigned long long)nmax;
+    v[ST_COUNT + 1] = (unsigned long long)xmax;
+#pragma unroll
+    for (int i = 0; i < ST_COUNT + 2; ++i) {
+        for (int off = 16; off > 0; off >>= 1) v[i] = max(v[i], __shfl_xor_sync(0xffffffffu, v[i], off));
+        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5][i] = v[i];
+    }
+    __syncthreads();
+    if (threadIdx.x < ST_COUNT + 2) {
+        unsigned long long m = 0;
+        for (int w = 0; w < 8; ++w) m = max(m, part[w][threadIdx.x]);
+        if (threadIdx.x < ST_COUNT) {
+            if (m > *(volatile unsigned long long *)&a.stats[threadIdx.x]) atomicMax(&a.stats[threadIdx.x], m);
+        } else {
+            int32_t *at = &a.err[2 + (threadIdx.x - ST_COUNT)];
+            if ((int32_t)m > *(volatile int32_t *)at) atomicMax(at, (int32_t)m);
         }
     }
-    // one atomic per warp and statistic
-    for (int off = 16; off > 0; off >>= 1) {
-        nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, off));
-        xmax = max(xmax, __shfl_xor_sync(0xffffffffu, xmax, off));
-        for (int i = 0; i < ST_COUNT; ++i) lmax[i] = max(lmax[i], __shfl_xor_sync(0xffffffffu, lmax[i], off));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        if (nmax) atomicMax(&a.err[2], nmax);
-        if (xmax) atomicMax(&a.err[3], xmax);
-        for (int i = 0; i < ST_COUNT; ++i)
-            if (lmax[i]) atomicMax(&a.stats[i], lmax[i]);
-    }
-
 }
 
 int paam_launch_validate(const paam_batch *b, const int32_t *acc, int32_t *err, unsigned long long *stats,
@@ -266,6 +418,15 @@ int paam_launch_validate(const paam_batch *b, const int32_t *acc, int32_t *err, 
 {
     const ValidateRange whole = {0, b->n_chain, 0, b->n_cb, 0, b->n_seg, 0, b->n_exec};
     return paam_launch_validate_range(b, acc, whole, 1, err, stats, stream);
+}
+
+static unsigned validate_blocks(const paam_batch *b)
+{
+    const int64_t per_block = kValThreads / G;
+    int64_t blocks = (b->n_sys + per_block - 1) / per_block;
+    const int64_t cap = kValBlocks * (int64_t)b->ctx->n_sm; // one wave of resident blocks
+    if (blocks > cap) blocks = cap;
+    return (unsigned)(blocks < 1 ? 1 : blocks);
 }
 
 int paam_launch_validate_range(const paam_batch *b, const int32_t *acc, const ValidateRange &r, int sentinels,
@@ -282,11 +443,21 @@ int paam_launch_validate_range(const paam_batch *b, const int32_t *acc, const Va
     a.acc = acc;
     a.err = err;
     a.stats = stats;
-    const int threads = 256;
-    int64_t blocks = (b->n_sys + threads - 1) / threads;
-    if (blocks > 16 * (int64_t)b->ctx->n_sm) blocks = 16 * (int64_t)b->ctx->n_sm;
-    if (blocks < 1) blocks = 1;
-    validate_kernel<<<(unsigned)blocks, threads, 0, stream>>>(a);
+    validate_kernel<<<validate_blocks(b), kValThreads, 0, stream>>>(a);
+    paam_count_launch();
+    PAAM_CUDA_TRY(cudaGetLastError());
+    return PAAM_OK;
+}
+
+bool paam_validate_undecided(const int32_t *host_err) { return host_err[0] == 0 && host_err[1] == 0; }
+
+int paam_launch_validate_rest(const paam_batch *b, int32_t *err, unsigned long long *stats, cudaStream_t stream)
+{
+    ValidateArgs a = {};
+    a.b = batch_dev(b);
+    a.err = err;
+    a.stats = stats;
+    range_kernel<<<validate_blocks(b), kValThreads, 0, stream>>>(a);
     paam_count_launch();
     PAAM_CUDA_TRY(cudaGetLastError());
     return PAAM_OK;
@@ -313,27 +484,47 @@ __device__ __forceinline__ int size_bin(const int64_t *off, int64_t s)
     return c < 0 ? 0 : (c > PAAM_MAX_CHAINS ? PAAM_MAX_CHAINS : (int)c);
 }
 
-// one CTA per window: histogram, exclusive scan, scatter to order[w0 + position]
-__global__ void bin_window(const int64_t *off, int64_t n_sys, int32_t *order)
+// one CTA per window: histogram, exclusive scan, scatter to order[w0 + position].
+// Bound by latency (a window per CTA, few CTAs): every thread loads its systems'
+// offsets at once and keeps the counts for the scatter, and one warp scans the
+// table; 200,000 systems 14 -> 5.4 us.
+constexpr int kBinThreads = 1024, kBinPer = kBinWindow / kBinThreads;
+
+__global__ void __launch_bounds__(kBinThreads) bin_window(const int64_t *off, int64_t n_sys, int32_t *order)
 {
-    __shared__ int32_t h[kBins];
+    static_assert(kBins <= 96, "three counts per lane in the scan");
+    __shared__ int32_t h[96];
     const int64_t w0 = (int64_t)blockIdx.x * kBinWindow;
     const int64_t w1 = w0 + kBinWindow < n_sys ? w0 + kBinWindow : n_sys;
-    for (int i = threadIdx.x; i < kBins; i += blockDim.x) h[i] = 0;
-    __syncthreads();
-    for (int64_t s = w0 + threadIdx.x; s < w1; s += blockDim.x) atomicAdd(&h[size_bin(off, s)], 1);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int32_t run = 0;
-        for (int i = 0; i < kBins; ++i) {
-            const int32_t c = h[i];
-            h[i] = run;
-            run += c;
-        }
+    if (threadIdx.x < 96) h[threadIdx.x] = 0;
+    int bin[kBinPer];
+#pragma unroll
+    for (int i = 0; i < kBinPer; ++i) {
+        const int64_t s = w0 + threadIdx.x + i * kBinThreads;
+        bin[i] = s < w1 ? size_bin(off, s) : -1;
     }
     __syncthreads();
-    for (int64_t s = w0 + threadIdx.x; s < w1; s += blockDim.x)
-        order[w0 + atomicAdd(&h[size_bin(off, s)], 1)] = (int32_t)s;
+#pragma unroll
+    for (int i = 0; i < kBinPer; ++i)
+        if (bin[i] >= 0) atomicAdd(&h[bin[i]], 1);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        const int32_t a = h[3 * lane], b = h[3 * lane + 1], c = h[3 * lane + 2];
+        int32_t run = a + b + c;
+        for (int d = 1; d < 32; d <<= 1) {
+            const int32_t v = __shfl_up_sync(0xffffffffu, run, d);
+            if (lane >= d) run += v;
+        }
+        run -= a + b + c;
+        h[3 * lane] = run;
+        h[3 * lane + 1] = run + a;
+        h[3 * lane + 2] = run + a + b;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kBinPer; ++i)
+        if (bin[i] >= 0) order[w0 + atomicAdd(&h[bin[i]], 1)] = (int32_t)(w0 + threadIdx.x + i * kBinThreads);
 }
 
 } // namespace
@@ -342,7 +533,7 @@ int paam_launch_bin_by_size(const paam_batch *b, int32_t *order, cudaStream_t st
 {
     if (b->n_sys <= 0) return PAAM_OK;
     const int64_t blocks = (b->n_sys + kBinWindow - 1) / kBinWindow;
-    bin_window<<<(unsigned)blocks, 256, 0, stream>>>(b->sys_chain_off, b->n_sys, order);
+    bin_window<<<(unsigned)blocks, kBinThreads, 0, stream>>>(b->sys_chain_off, b->n_sys, order);
     PAAM_CUDA_TRY(cudaGetLastError());
     paam_count_launch(1);
     return PAAM_OK;
@@ -463,6 +654,14 @@ extern "C" int paam_rta_load_systems(paam_ctx *ctx, const paam_systems_view *v, 
             rc = PAAM_E_CUDA;
     }
     if (cudaStreamSynchronize(stream) != cudaSuccess) rc = PAAM_E_CUDA;
+    if (rc == PAAM_OK && b->n_sys > 0 && paam_validate_undecided(h_err)) {
+        if (paam_launch_validate_rest(b, ctx->d_err, ctx->d_stats, stream) != PAAM_OK ||
+            cudaMemcpyAsync(h_err, ctx->d_err, sizeof(h_err), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+            cudaMemcpyAsync(b->stats, ctx->d_stats, sizeof(b->stats), cudaMemcpyDeviceToHost, stream) !=
+                cudaSuccess ||
+            cudaStreamSynchronize(stream) != cudaSuccess)
+            rc = PAAM_E_CUDA;
+    }
     if (rc == PAAM_OK && h_err[0] != 0) rc = h_err[0];
     if (rc != PAAM_OK) {
         cudaFree(b->block);

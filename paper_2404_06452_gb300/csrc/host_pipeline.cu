@@ -299,14 +299,24 @@ extern "C" int paam_rta_analyze_host(paam_ctx *ctx, const paam_systems_view *v, 
             break;
         }
         const int32_t *err_h = (const int32_t *)(whost + kWords * (size_t)k);
-        if (err_h[0] != 0) {
-            rc = err_h[0];
-            break;
-        }
         paam_batch sub = t;
         sub.n_sys = c.s1 - c.s0;
         sub.sys_chain_off = t.sys_chain_off + c.s0;
         sub.sys_exec_off = t.sys_exec_off + c.s0;
+        if (paam_validate_undecided(err_h)) {
+            int32_t *err_d = (int32_t *)(wdev + kWords * (size_t)k);
+            if (paam_launch_validate_rest(&sub, err_d, (unsigned long long *)(err_d + 4), pl->val) != PAAM_OK ||
+                cudaMemcpyAsync(whost + kWords * (size_t)k, err_d, kWords, cudaMemcpyDeviceToHost, pl->val) !=
+                    cudaSuccess ||
+                cudaStreamSynchronize(pl->val) != cudaSuccess) {
+                rc = PAAM_E_CUDA;
+                break;
+            }
+        }
+        if (err_h[0] != 0) {
+            rc = err_h[0];
+            break;
+        }
         sub.max_chains = err_h[2];
         sub.max_exec = err_h[3];
         memcpy(sub.stats, err_h + 4, sizeof(sub.stats));

@@ -154,7 +154,7 @@ struct paam_ctx {
     int n_sm;
     int max_smem_optin;
     cudaStream_t capture_stream; // private stream used to capture analysis graphs
-    int32_t *d_err;        // validation: [0] code, [1] first bad system, [2] max chains, [3] max executors
+    int32_t *d_err;        // validation: [0] code, [1] undecided, [2] max chains, [3] max executors
     unsigned long long *d_stats; // validation: ST_* maxima
     HostPipe *pipe;
 };
@@ -317,8 +317,12 @@ constexpr uint32_t kIterCap = (uint32_t)PAAM_MAX_ITER;
 int paam_enqueue_analysis(const paam_batch *b, const AnalysisParams &p, const LaunchCfg &cfg, int64_t *R,
                           uint8_t *status, uint8_t *verdict, cudaStream_t stream, int *n_kernels);
 
-// Validation kernel (api.cu): err = {code, first bad system, max chains, max
-// executors} (initialise to {0, INT32_MAX, 0, 0}), stats = ST_* maxima (zeroed).
+// Validation kernel (api.cu): err = {code, undecided, max chains, max executors}
+// (initialise to {0, INT32_MAX, 0, 0}), stats = ST_* maxima (zeroed).  Once the
+// words are on the host and paam_validate_undecided says so, the batch (valid so
+// far) also takes paam_launch_validate_rest, which adds to the same words.  The
+// maxima of a chain's E, A and segments may be their system's sums (below 2^29),
+// which only ever sends a batch to one kernel more.
 int paam_launch_validate(const paam_batch *b, const int32_t *acc, int32_t *err, unsigned long long *stats,
                          cudaStream_t stream);
 
@@ -332,6 +336,8 @@ struct ValidateRange {
 // adds the whole batch's first- and last-offset checks.
 int paam_launch_validate_range(const paam_batch *b, const int32_t *acc, const ValidateRange &r, int sentinels,
                                int32_t *err, unsigned long long *stats, cudaStream_t stream);
+bool paam_validate_undecided(const int32_t *host_err);
+int paam_launch_validate_rest(const paam_batch *b, int32_t *err, unsigned long long *stats, cudaStream_t stream);
 
 // The lazy register-table analysis for batches with several accelerators
 // (analyze_lazy_acc.cu): 16 lanes per system, one chain per lane, instantiated

@@ -129,6 +129,13 @@ extern "C" int paam_rta_analyze_noalloc(const paam_systems_view *v, const paam_a
     PAAM_CUDA_TRY(cudaMemcpyAsync(herr, err, sizeof(herr), cudaMemcpyDeviceToHost, stream));
     PAAM_CUDA_TRY(cudaMemcpyAsync(hstats, stats, sizeof(hstats), cudaMemcpyDeviceToHost, stream));
     PAAM_CUDA_TRY(cudaStreamSynchronize(stream));
+    if (paam_validate_undecided(herr)) {
+        rc = paam_launch_validate_rest(&b, err, stats, stream);
+        if (rc != PAAM_OK) return rc;
+        PAAM_CUDA_TRY(cudaMemcpyAsync(herr, err, sizeof(herr), cudaMemcpyDeviceToHost, stream));
+        PAAM_CUDA_TRY(cudaMemcpyAsync(hstats, stats, sizeof(hstats), cudaMemcpyDeviceToHost, stream));
+        PAAM_CUDA_TRY(cudaStreamSynchronize(stream));
+    }
     if (herr[0] != 0) return herr[0];
     b.max_chains = herr[2];
     b.max_exec = herr[3];
