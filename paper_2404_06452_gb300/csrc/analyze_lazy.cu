@@ -26,7 +26,7 @@
 // (blocking_mode 0) in analysis, candidate and target mode, and the safe reading
 // (blocking_mode 1, 16 lanes; its larger systems go to the int64 kernel); several
 // accelerators keep their kernel (analyze_lazy_acc.cu).
-#include "reg_common.cuh"
+#include "cand_eval.cuh"
 
 namespace {
 using namespace paam_reg;
@@ -681,16 +681,28 @@ __global__ void __launch_bounds__(256) chain_records_kernel(BatchDev b, uint64_t
             const unsigned sp = b.spin[g] != 0 ? 1u : 0u;
             // the chains of the same executor and of the same core (systems of up to 32
             // chains, the ones the lazy kernels read records for)
-            uint32_t sx = 0, sc = 0;
+            uint32_t sx = 0, sc = 0, fl = (a.fit ? paam_cand::kRecFit : 0u) | (sp ? paam_cand::kRecSpin : 0u);
             if (n <= 32) {
+                using namespace paam_cand;
                 const unsigned act = n == 32 ? 0xffffffffu : (1u << n) - 1u; // lanes j < n
                 sx = __match_any_sync(act, ex);
                 sc = __match_any_sync(act, co);
+                // the system's flags, the same in each of its records
+                const bool fit = __all_sync(act, a.fit != 0);
+                const uint32_t dmax = __reduce_max_sync(act, a.D);
+                // the iteration bound (lazy_system above)
+                const uint32_t arr = fit ? umin(rarrivals(dmax, a.tm2, a.mg, a.lg) - 1u, kIterCap + 1u) : 0u;
+                const uint32_t L = __reduce_add_sync(act, arr) + 2u;
+                const bool shared = __any_sync(act, (sc & (sc - 1u)) != 0);
+                const bool two = __any_sync(act, (sc & ~sx) != 0);
+                fl = (fit ? kRecFit : 0u) | (sp ? kRecSpin : 0u) | (fit && dmax < kNarrow - 16 ? kRecNarrow16 : 0u) |
+                     (fit && dmax < kNarrow - 32 ? kRecNarrow32 : 0u) | (L > kIterCap ? kRecCounted : 0u) |
+                     (shared ? kRecShared : 0u) | (two ? kRecTwoExec : 0u);
             }
             uint4 *r = recs + g * 4;
             r[0] = make_uint4(a.tm2, a.mg, a.lg, a.D);
             r[1] = make_uint4(a.E, a.S, a.Emax, a.M);
-            r[2] = make_uint4(a.Amin, a.dl, (uint32_t)(a.q0 - seg_base), a.fit | (sp << 1));
+            r[2] = make_uint4(a.Amin, a.dl, (uint32_t)(a.q0 - seg_base), fl);
             r[3] = make_uint4((uint32_t)ex, (uint32_t)co, sx, sc);
         }
     }
@@ -715,9 +727,10 @@ int launch_lazy_pass(const paam_batch *bt, const AnalysisParams &p, int64_t *R, 
                      const int32_t *list, const int32_t *count, int64_t max_items, int threads, cudaStream_t stream)
 {
     if (threads % 32 != 0 || threads > 256) return PAAM_E_INVAL;
+    if (p.chain_recs) return launch_cand<LG>(bt, p, list, count, max_items, stream);
     const int groups = threads / LG;
     const size_t smem = sizeof(LazySmem<LG>) * groups;
-    auto kern = p.chain_recs ? analyze_lazy_kernel<LG, BLOCKS, true> : analyze_lazy_kernel<LG, BLOCKS, false>;
+    auto kern = analyze_lazy_kernel<LG, BLOCKS, false>;
     PAAM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     PAAM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));

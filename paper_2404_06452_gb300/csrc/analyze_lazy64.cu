@@ -434,6 +434,25 @@ __device__ void lazy64_system(const BatchDev &b, const AnalysisParams &p, int64_
     }
 
     // ---- own recurrence terms ------------------------------------------------
+    if (rank_row) {
+        // a candidate with a chain whose R is above its deadline whatever its
+        // interference's arrivals (the bound of cand_eval.cuh) fails at once
+        bool over = false;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint64_t f = ((uint64_t)Amn[k] + blk[k]) >= 1 ? 2 : 1;
+            const uint64_t low = (uint64_t)Bv[k] + Ev[k] +
+                                 (user[k] ? (uint64_t)Sv[k] + (uint64_t)dlv[k] * blk[k] + (uint64_t)dlv[k] * eps +
+                                                f * sums[k]
+                                          : 0);
+            over |= val[k] && low > Dv[k];
+        }
+        if (__any_sync(kFull, over)) {
+            if (lane == 0 && p.cand_ok) p.cand_ok[sys * p.Kc + cand_of(p, sys, cand)] = 0;
+            __syncwarp();
+            return;
+        }
+    }
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         if (!val[k]) continue;

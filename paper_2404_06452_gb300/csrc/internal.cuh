@@ -282,6 +282,11 @@ int launch_lazy32(const paam_batch *bt, const AnalysisParams &p, int64_t *R, uin
 // that are not narrow (a deadline at or above kLazyDeferWideD) go to b->list_wide.
 int launch_lazy64(const paam_batch *bt, const AnalysisParams &p, int64_t *R, uint8_t *st, uint8_t *verdict,
                   const int32_t *list, const int32_t *count, int64_t max_items, int threads, cudaStream_t stream);
+// The candidate mode with chain records (analyze_cand.cu), LG = 16 (every item)
+// or 32 (the deferral list); deferred items as the lazy passes defer them.
+template <int LG>
+int launch_cand(const paam_batch *bt, const AnalysisParams &p, const int32_t *list, const int32_t *count,
+                int64_t max_items, cudaStream_t stream);
 // The per-chain records of AnalysisParams::chain_recs for every chain of b
 // (analyze_lazy.cu): the aggregates the lazy kernels compute before the
 // relations, which do not depend on the priorities.
