@@ -547,6 +547,14 @@ LaunchFn find_variant(int impl, int G, int maxn)
 
 } // namespace
 
+bool paam_batch_fits_32(const paam_batch *b, const paam_analysis_opts *o)
+{
+    AnalysisParams p = {};
+    p.eps = o->eps_ns;
+    p.kappa = o->kappa_ns;
+    return batch_fits_32(b, p);
+}
+
 // Candidate launch configurations the autotuner times (kDefaultLaunchCfg is
 // the one a batch starts with).
 const LaunchCfg kLaunchCfgs[] = {

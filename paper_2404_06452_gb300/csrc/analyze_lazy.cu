@@ -136,17 +136,13 @@ __device__ __forceinline__ void chain_aggregates(const BatchDev &b, int64_t g, u
     a.q0 = q0;
 }
 
-// REC: the aggregates come from p.chain_recs (candidate mode).  TGT (target mode,
-// the Audsley-style seed; see AnalysisParams.target): candidate (system, c) is
-// decided by chain p.target[system * Kc + c] alone (-1: no trial in the slot), the
-// chains are analysed up to that one's step and no failure ends a candidate early.
-// SAFE (16 lanes, aggregates computed here): the safe reading of Lemma 4
+// SAFE (16 lanes): the safe reading of Lemma 4
 // (blocking_mode 1): every segment's Lemma 2 bound is computed (one segment per
 // lane), each chain's longest callback hold E_i + sum over its segments of (bound
 // + eps), B_c as the longest hold of a lower-priority chain on c's executor, and
 // Eq. 3's exact sum in every recurrence; systems of more than kSafeSegs segments
 // go to the int64 kernel's list.
-template <int LG, bool REC = false, bool TGT = false, bool SAFE = false>
+template <int LG, bool SAFE = false>
 __device__ void lazy_system(const BatchDev &b, const AnalysisParams &p, int64_t item, LazySmem<LG> &s,
                             LazySafeExt<LG> *sx, int lane,
                             unsigned gm, int64_t *__restrict__ R_out, uint8_t *__restrict__ st_out,
@@ -163,11 +159,6 @@ __device__ void lazy_system(const BatchDev &b, const AnalysisParams &p, int64_t 
     }
     const int64_t c0 = b.sys_chain_off[sys];
     const int n = (int)(b.sys_chain_off[sys + 1] - c0);
-    int tgt = -1;
-    if constexpr (TGT) {
-        tgt = p.target[sys * p.Kc + cand_of(p, sys, cand)];
-        if (tgt < 0 || tgt >= n) return; // no trial in this slot
-    }
     if (n > LG) { // the 64-chain kernel's; the first pass appends it to its list
         if (LG == 16 && lane == 0) big_list[atomicAdd(big_count, 1)] = (int32_t)item;
         return;
@@ -186,7 +177,6 @@ __device__ void lazy_system(const BatchDev &b, const AnalysisParams &p, int64_t 
     bool sp = false;
     unsigned fit = 1, rank_ok = 1;
     Mask rbit = 0;
-    uint32_t rsx = 0, rco = 0; // same-executor and same-core chains, from the records
     const bool val = j < n;
     if (val) {
         const int64_t g = c0 + j;
@@ -198,33 +188,22 @@ __device__ void lazy_system(const BatchDev &b, const AnalysisParams &p, int64_t 
         } else {
             pr = b.prio[g];
         }
-        if constexpr (REC) {
-            const uint4 *r = p.chain_recs + g * 4;
-            const uint4 r0 = r[0], r1 = r[1], r2 = r[2], r3 = r[3];
-            tm2 = r0.x, mg = r0.y, lg = r0.z, Dv = r0.w;
-            Ev = r1.x, Sv = r1.y, Emx = r1.z, Mv = r1.w;
-            Amn = r2.x, dlv = r2.y, seg0 = r2.z, fit = r2.w & 1u, sp = (r2.w >> 1) & 1u;
-            ex = (int32_t)r3.x, co = (int32_t)r3.y;
-            rsx = r3.z, rco = r3.w;
-            if (xprio) ep = xprio[x0 + ex];
-        } else {
-            ex = b.exec[g];
-            co = b.exec_core[x0 + ex];
-            if (xprio) ep = xprio[x0 + ex];
-            sp = b.spin[g] != 0;
-            ChainAgg a;
-            chain_aggregates(b, g, kappa2, eps, a);
-            fit = a.fit;
-            tm2 = a.tm2, mg = a.mg, lg = a.lg;
-            Dv = a.D;
-            Ev = a.E;
-            Sv = a.S;
-            Emx = a.Emax;
-            Mv = a.M;
-            Amn = a.Amin;
-            dlv = a.dl;
-            seg0 = (uint32_t)(a.q0 - seg_base);
-        }
+        ex = b.exec[g];
+        co = b.exec_core[x0 + ex];
+        if (xprio) ep = xprio[x0 + ex];
+        sp = b.spin[g] != 0;
+        ChainAgg a;
+        chain_aggregates(b, g, kappa2, eps, a);
+        fit = a.fit;
+        tm2 = a.tm2, mg = a.mg, lg = a.lg;
+        Dv = a.D;
+        Ev = a.E;
+        Sv = a.S;
+        Emx = a.Emax;
+        Mv = a.M;
+        Amn = a.Amin;
+        dlv = a.dl;
+        seg0 = (uint32_t)(a.q0 - seg_base);
     }
     if (lane == 0) {
         s.c0 = c0;
@@ -277,17 +256,8 @@ __device__ void lazy_system(const BatchDev &b, const AnalysisParams &p, int64_t 
     const bool counted = L > kIterCap;
 
     // ---- relations (Lemma 4, Theorem 1, Eq. 3), analysis order ---------------
-    // lanes of the same executor (unique keys past n) and of the same core: from the
-    // chain records (every lane of the group takes the same path), or matched here
-    unsigned xm;
-    Mask corem;
-    if constexpr (REC) {
-        xm = (val ? rsx : jbit) << sh;
-        corem = val ? rco : jbit;
-    } else {
-        xm = __match_any_sync(gm, ex);
-        corem = __match_any_sync(gm, co) >> sh;
-    }
+    const unsigned xm = __match_any_sync(gm, ex); // lanes of the same executor (unique keys past n)
+    const Mask corem = __match_any_sync(gm, co) >> sh;
     const Mask samex = xm >> sh;
     if (!xprio) ep = __reduce_max_sync(xm, pr); // criticality-as-priority: highest chain priority on the executor
     const bool one_bucket = p.n_buckets == 1;
@@ -484,12 +454,10 @@ __device__ void lazy_system(const BatchDev &b, const AnalysisParams &p, int64_t 
     const uint32_t k2 = (uint32_t)kappa2;
     auto chains = [&](auto counted_tag) {
     constexpr bool CNT = decltype(counted_tag)::value;
-    // target mode: up to the target chain's step
-    const int nsteps = TGT ? __shfl_sync(gm, pos, tgt, LG) + 1 : n;
-    for (int step = 0; step < nsteps; ++step) {
+    for (int step = 0; step < n; ++step) {
         const uint4 rl = s.rel[step];
         if (rl.w & ~sched) { // a needed H*_h is not available (the chain is DEP)
-            if (rank_row && !TGT) break; // a candidate fails at its first unschedulable chain
+            if (rank_row) break; // a candidate fails at its first unschedulable chain
             continue;
         }
         const uint4 rc = s.rec[step], sg = s.seg[step];
@@ -501,7 +469,7 @@ __device__ void lazy_system(const BatchDev &b, const AnalysisParams &p, int64_t 
         const uint32_t dl = sg.w;
         if (SAFE && dl && sg.y == kCapR) { // a segment recurrence was cut short: no bound (PAAM_ST_ITERCAP)
             if (j == c) Rv = kCapR;
-            if (rank_row && !TGT) break;
+            if (rank_row) break;
             continue;
         }
         // start: B + E + H* with the interference part of Eq. 4 empty; Lemma 2's sum is
@@ -577,7 +545,7 @@ __device__ void lazy_system(const BatchDev &b, const AnalysisParams &p, int64_t 
         }
         if (capped) { // no bound (PAAM_ST_ITERCAP)
             if (j == c) Rv = kCapR;
-            if (rank_row && !TGT) break;
+            if (rank_row) break;
             continue;
         }
         if (ok) {
@@ -589,7 +557,7 @@ __device__ void lazy_system(const BatchDev &b, const AnalysisParams &p, int64_t 
             }
         } else {
             if (ev > kIterCap && j == c) Rv = kCapR; // the recurrence was cut short (PAAM_ST_ITERCAP)
-            if (rank_row && !TGT) break;
+            if (rank_row) break;
         }
     }
     };
@@ -602,11 +570,6 @@ __device__ void lazy_system(const BatchDev &b, const AnalysisParams &p, int64_t 
     {
     const int64_t c0 = s.c0, sys = s.sys;
     const int32_t cand = s.cand;
-    if (TGT) { // the target chain's verdict; first_ok is not touched
-        if (lane == 0) p.cand_ok[sys * p.Kc + cand_of(p, sys, cand)] = ((sched >> tgt) & 1) ? 1 : 0;
-        __syncwarp(gm);
-        return;
-    }
     if (rank_row) {
         if (lane == 0) {
             const bool ok = sched == all;
@@ -631,7 +594,7 @@ __device__ void lazy_system(const BatchDev &b, const AnalysisParams &p, int64_t 
 
 // BLOCKS resident blocks of 256 threads per SM: the register budget per thread.
 // Items are all of the launch (list == nullptr) or list[0 .. *count).
-template <int LG, int BLOCKS, bool REC, bool TGT = false, bool SAFE = false>
+template <int LG, int BLOCKS, bool SAFE = false>
 __global__ void __launch_bounds__(256, BLOCKS) analyze_lazy_kernel(BatchDev b, AnalysisParams p, int64_t *R,
                                                                    uint8_t *st, uint8_t *verdict, const int32_t *list,
                                                                    const int32_t *count, int32_t *big_list,
@@ -656,13 +619,14 @@ __global__ void __launch_bounds__(256, BLOCKS) analyze_lazy_kernel(BatchDev b, A
         if (!list && p.K == 0 && lane == 0 && i % kPrefetchSlice == 0)
             prefetch_systems(b, p.sys_order, i + kBinWindow, kPrefetchSlice);
         const int64_t item = list ? (int64_t)list[i] : i;
-        lazy_system<LG, REC, TGT, SAFE>(b, p, item, s, sx, lane, gm, R, st, verdict, big_list, big_count, wide_list,
+        lazy_system<LG, SAFE>(b, p, item, s, sx, lane, gm, R, st, verdict, big_list, big_count, wide_list,
                                         wide_count);
     });
 }
 
 // one warp per system, one lane per chain: the records of chain_recs
-__global__ void __launch_bounds__(256) chain_records_kernel(BatchDev b, uint64_t kappa2, uint64_t eps, uint4 *recs)
+__global__ void __launch_bounds__(256) chain_records_kernel(BatchDev b, uint64_t kappa2, uint64_t eps, uint4 *recs,
+                                                            int32_t rec_stride)
 {
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -699,7 +663,7 @@ __global__ void __launch_bounds__(256) chain_records_kernel(BatchDev b, uint64_t
                      (fit && dmax < kNarrow - 32 ? kRecNarrow32 : 0u) | (L > kIterCap ? kRecCounted : 0u) |
                      (shared ? kRecShared : 0u) | (two ? kRecTwoExec : 0u);
             }
-            uint4 *r = recs + g * 4;
+            uint4 *r = recs + (rec_stride ? sys * rec_stride + j : g) * 4;
             r[0] = make_uint4(a.tm2, a.mg, a.lg, a.D);
             r[1] = make_uint4(a.E, a.S, a.Emax, a.M);
             r[2] = make_uint4(a.Amin, a.dl, (uint32_t)(a.q0 - seg_base), fl);
@@ -710,13 +674,14 @@ __global__ void __launch_bounds__(256) chain_records_kernel(BatchDev b, uint64_t
 
 } // namespace
 
-int paam_launch_chain_records(const paam_batch *bt, const AnalysisParams &p, uint4 *recs, cudaStream_t stream)
+int paam_launch_chain_records(const paam_batch *bt, const AnalysisParams &p, uint4 *recs, cudaStream_t stream,
+                              int32_t rec_stride)
 {
     if (bt->n_sys <= 0) return PAAM_OK;
     int64_t blocks = (bt->n_sys + 7) / 8;
     if (blocks > 16 * (int64_t)bt->ctx->n_sm) blocks = 16 * (int64_t)bt->ctx->n_sm;
     chain_records_kernel<<<(unsigned)blocks, 256, 0, stream>>>(batch_dev(bt), 2 * (uint64_t)p.kappa,
-                                                               (uint64_t)p.eps, recs);
+                                                               (uint64_t)p.eps, recs, rec_stride);
     PAAM_CUDA_TRY(cudaGetLastError());
     paam_count_launch();
     return PAAM_OK;
@@ -730,7 +695,7 @@ int launch_lazy_pass(const paam_batch *bt, const AnalysisParams &p, int64_t *R, 
     if (p.chain_recs) return launch_cand<LG>(bt, p, list, count, max_items, stream);
     const int groups = threads / LG;
     const size_t smem = sizeof(LazySmem<LG>) * groups;
-    auto kern = analyze_lazy_kernel<LG, BLOCKS, false>;
+    auto kern = analyze_lazy_kernel<LG, BLOCKS>;
     PAAM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     PAAM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
@@ -751,7 +716,7 @@ int paam_launch_lazy_safe(const paam_batch *bt, const AnalysisParams &p, int64_t
     constexpr int LG = 16, threads = 256;
     const int groups = threads / LG;
     const size_t smem = sizeof(LazySafeSmem<LG>) * groups;
-    auto kern = analyze_lazy_kernel<LG, 5, false, false, true>;
+    auto kern = analyze_lazy_kernel<LG, 5, true>;
     PAAM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     PAAM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
@@ -764,28 +729,6 @@ int paam_launch_lazy_safe(const paam_batch *bt, const AnalysisParams &p, int64_t
     // outside the 32-bit bound) to the int64 kernel's list
     kern<<<(unsigned)blocks, threads, smem, stream>>>(batch_dev(bt), p, R, st, verdict, nullptr, nullptr,
                                                       bt->list_wide, bt->counts + 1, bt->list_wide, bt->counts + 1);
-    PAAM_CUDA_TRY(cudaGetLastError());
-    return PAAM_OK;
-}
-
-int paam_launch_lazy_target(const paam_batch *bt, const AnalysisParams &p, int32_t *list, int32_t *count,
-                            int64_t max_items, cudaStream_t stream)
-{
-    constexpr int LG = 16, threads = 256;
-    const int groups = threads / LG;
-    const size_t smem = sizeof(LazySmem<LG>) * groups;
-    auto kern = p.chain_recs ? analyze_lazy_kernel<LG, 5, true, true> : analyze_lazy_kernel<LG, 5, false, true>;
-    PAAM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int per_sm = 0;
-    PAAM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
-    if (per_sm < 1) per_sm = 1;
-    int64_t blocks = (max_items + groups - 1) / groups;
-    const int64_t cap = (int64_t)per_sm * bt->ctx->n_sm;
-    if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
-    // every deferred trial (over 16 chains, not narrow, outside the 32-bit bound) to list
-    kern<<<(unsigned)blocks, threads, smem, stream>>>(batch_dev(bt), p, nullptr, nullptr, nullptr, nullptr, nullptr,
-                                                      list, count, list, count);
     PAAM_CUDA_TRY(cudaGetLastError());
     return PAAM_OK;
 }

@@ -61,7 +61,7 @@ struct AnalysisParams {
     // sys_order[k] (systems sorted by chain count), so the groups that share a
     // warp analyse systems of one size and stay converged longer.
     const int32_t *sys_order;
-    // Target mode (the Audsley-style seed; the int64 and lazy kernels): with
+    // Target mode (the Audsley-style seed; the int64 kernel): with
     // target set, candidate (system, c) is decided by one chain,
     // target[system * Kc + c] (-1: skip the item): cand_ok receives whether
     // that chain is schedulable, the analysis stops once it is done, and
@@ -290,7 +290,11 @@ int launch_cand(const paam_batch *bt, const AnalysisParams &p, const int32_t *li
 // The per-chain records of AnalysisParams::chain_recs for every chain of b
 // (analyze_lazy.cu): the aggregates the lazy kernels compute before the
 // relations, which do not depend on the priorities.
-int paam_launch_chain_records(const paam_batch *b, const AnalysisParams &p, uint4 *recs, cudaStream_t stream);
+// rec_stride 0: the records in chain order; else system s's at s * rec_stride.
+int paam_launch_chain_records(const paam_batch *b, const AnalysisParams &p, uint4 *recs, cudaStream_t stream,
+                              int32_t rec_stride = 0);
+// Every system of the batch is inside the 32-bit bound under these overheads.
+bool paam_batch_fits_32(const paam_batch *b, const paam_analysis_opts *o);
 // impl_big value of a launch configuration whose deferral list goes to the 32-lane
 // lazy kernel and then, for systems over 32 chains, to the 64-chain lazy kernel
 constexpr int kImplBigLazy32 = 9;
@@ -353,7 +357,7 @@ int paam_launch_lazy_acc(const paam_batch *bt, const AnalysisParams &p, int64_t 
                          int64_t max_items, cudaStream_t stream);
 
 
-// Chains up to which a search (or the Audsley-style seed) keeps each chain's
+// Chains up to which a search keeps each chain's
 // aggregates for all its candidates (paam_launch_chain_records, 64 bytes per chain).
 constexpr int64_t kRecChains = (int64_t)1 << 22;
 
@@ -362,13 +366,6 @@ constexpr int64_t kRecChains = (int64_t)1 << 22;
 // accelerator; the others are appended to b->list_wide (count b->counts[1]).
 int paam_launch_lazy_safe(const paam_batch *bt, const AnalysisParams &p, int64_t *R, uint8_t *st, uint8_t *verdict,
                           int64_t max_items, cudaStream_t stream);
-
-// Target mode of the lazy kernel (analyze_lazy.cu), reading p.chain_recs when set:
-// candidates of systems with up to 16 chains inside the narrow 32-bit bound, one
-// accelerator, Lemma 4 as printed; the others are appended to list (count *count)
-// for the int64 kernel.
-int paam_launch_lazy_target(const paam_batch *bt, const AnalysisParams &p, int32_t *list, int32_t *count,
-                            int64_t max_items, cudaStream_t stream);
 
 // Exact int64 kernel (analyze_wide.cu) over list[0 .. *count) or, with
 // list == nullptr, over every system.

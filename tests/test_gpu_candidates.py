@@ -1,5 +1,5 @@
-"""GPU parity of the candidate verdicts (the search) at the edges of their group
-widths, with shared and unshared executors and
+"""GPU parity of the candidate verdicts (the search) and of the Audsley-style
+seed at the edges of their group widths, with shared and unshared executors and
 cores, busy-waiting chains, several buckets and both blocking readings' options
 left to the other kernels, against the CPU oracle."""
 from __future__ import annotations
@@ -54,6 +54,30 @@ def test_search_verdicts(shape, util):
         seen |= set(np.unique(ref["cand_ok"]))
     if util < 0.1:
         assert seen == {0, 1}  # both verdicts occur
+
+
+@pytest.mark.parametrize("shape", list(SHAPES))
+def test_seed_order(shape):
+    import paper_2404_06452_gb300 as pkg
+
+    for p in PARAMS[:3]:
+        sy = _batch(shape, 40, 0.3)
+        nmax = int(sy.chains_per_system().max()) + 1
+        b = pkg.paam_rta_load_systems(ctx(), sy)
+        got = pkg.audsley_order(ctx(), b, nmax, **p).cpu().numpy()
+        assert np.array_equal(got, oracle.audsley(sy, nmax=nmax, threads=8, **p)), p
+
+
+@pytest.mark.parametrize("n_sys", [608, 609, 4865])
+def test_seed_order_batch_sizes(n_sys):
+    """Each number of groups per system."""
+    import paper_2404_06452_gb300 as pkg
+
+    cfg = dict(paam_gen.CONFIGS["cfg4s"], n_min=2, n_max=9, x_min=2, x_max=9, exec_per_core=2)
+    sy = paam_gen.generate(cfg, n_sys=n_sys)
+    b = pkg.paam_rta_load_systems(ctx(), sy)
+    got = pkg.audsley_order(ctx(), b, 9, n_buckets=2).cpu().numpy()
+    assert np.array_equal(got, oracle.audsley(sy, nmax=9, n_buckets=2, threads=8))
 
 
 def test_short_periods_take_the_joint_evaluation_past_its_limit():
