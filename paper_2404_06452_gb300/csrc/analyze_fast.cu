@@ -611,17 +611,37 @@ int paam_enqueue_analysis(const paam_batch *b, const AnalysisParams &p, const La
         pw.queue = b->queue + 2;
         pm.queue_batch = pb.queue_batch = pw.queue_batch = cfg.queue;
     }
-    if (p.blocking_mode == 1) { // the safe blocking term in the lazy kernel, the int64 kernel for the rest
-        int rc = paam_launch_lazy_safe(b, pm, R, status, verdict, items, stream);
-        if (rc == PAAM_OK) rc = paam_launch_wide(b, pw, R, status, verdict, b->list_wide, b->counts + 1, items, stream);
-        if (n_kernels) *n_kernels = 2;
-        return rc;
-    }
-    if (b->acc) { // several accelerators: per-accelerator register tables, the int64 kernel for the rest
-        int rc = paam_launch_lazy_acc(b, pm, R, status, verdict, items, stream);
-        if (rc == PAAM_OK) rc = paam_launch_wide(b, pw, R, status, verdict, b->list_wide, b->counts + 1, items, stream);
-        if (n_kernels) *n_kernels = 2;
-        return rc;
+    if (p.blocking_mode == 1 || b->acc) {
+        // the safe blocking term, or several accelerators: their 16-lane kernels, then
+        // one warp per larger system, each pass only where the batch has systems for it
+        int rc = p.blocking_mode == 1 ? paam_launch_lazy_safe(b, pm, R, status, verdict, items, stream)
+                                      : paam_launch_lazy_acc(b, pm, R, status, verdict, items, stream);
+        if (rc != PAAM_OK) return rc;
+        ++k;
+        const bool safe = p.blocking_mode == 1, fits = batch_fits_32(b, p);
+        if (b->max_chains > 16 ||
+            (safe && (b->stats[ST_SEGMAX] > kSafeSegs || b->stats[ST_DMAX] >= kLazyNarrowD))) {
+            rc = paam_launch_lazy_big(b, 1, pb, R, status, verdict, items, stream);
+            if (rc != PAAM_OK) return rc;
+            ++k;
+        }
+        if (b->max_chains > 32) {
+            AnalysisParams ph = pb;
+            if (pb.queue_batch > 0) { // the first pass's counter, reset: that pass is done
+                PAAM_CUDA_TRY(cudaMemsetAsync(b->queue, 0, sizeof(unsigned long long), stream));
+                ph.queue = b->queue;
+            }
+            rc = paam_launch_lazy_big(b, 2, ph, R, status, verdict, items, stream);
+            if (rc != PAAM_OK) return rc;
+            ++k;
+        }
+        if (!fits || b->stats[ST_DMAX] >= kLazyDeferWideD || (safe && b->stats[ST_SEGMAX] > kBigSegs)) {
+            rc = paam_launch_wide(b, pw, R, status, verdict, b->list_wide, b->counts + 1, items, stream);
+            if (rc != PAAM_OK) return rc;
+            ++k;
+        }
+        if (n_kernels) *n_kernels = k;
+        return PAAM_OK;
     }
     int rc = small(b, pm, R, status, verdict, nullptr, nullptr, items, cfg.threads, stream);
     if (rc != PAAM_OK) return rc;

@@ -24,8 +24,9 @@
 // then analyze_lazy64.cu for those above 32 chains); systems outside the 32-bit
 // bound to b.list_wide (the int64 kernel).  One accelerator: Lemma 4 as printed
 // (blocking_mode 0) in analysis, candidate and target mode, and the safe reading
-// (blocking_mode 1, 16 lanes; its larger systems go to the int64 kernel); several
-// accelerators keep their kernel (analyze_lazy_acc.cu).
+// (blocking_mode 1, 16 lanes); several accelerators keep their kernel
+// (analyze_lazy_acc.cu), and the larger systems of both options theirs
+// (analyze_lazy_big.cu).
 #include "cand_eval.cuh"
 
 namespace {
@@ -59,7 +60,6 @@ struct LazySmem {
 
 // The safe reading of Lemma 4 (blocking_mode 1) also bounds every segment of the
 // system, one per lane, from these tables (systems of up to kSafeSegs segments).
-constexpr int kSafeSegs = 128;
 template <int LG>
 struct LazySafeExt {
     uint4 dv[LG];             // by chain: {2 (T - 1), magic, l, S*} (the interferer's term)
@@ -141,7 +141,7 @@ __device__ __forceinline__ void chain_aggregates(const BatchDev &b, int64_t g, u
 // lane), each chain's longest callback hold E_i + sum over its segments of (bound
 // + eps), B_c as the longest hold of a lower-priority chain on c's executor, and
 // Eq. 3's exact sum in every recurrence; systems of more than kSafeSegs segments
-// go to the int64 kernel's list.
+// go to the deferral list.
 template <int LG, bool SAFE = false>
 __device__ void lazy_system(const BatchDev &b, const AnalysisParams &p, int64_t item, LazySmem<LG> &s,
                             LazySafeExt<LG> *sx, int lane,
@@ -242,7 +242,7 @@ __device__ void lazy_system(const BatchDev &b, const AnalysisParams &p, int64_t 
     if constexpr (SAFE) {
         nseg = __reduce_add_sync(gm, val ? dlv : 0u);
         if (nseg > (uint32_t)kSafeSegs) {
-            if (lane == 0) wide_list[atomicAdd(wide_count, 1)] = (int32_t)item;
+            if (lane == 0) big_list[atomicAdd(big_count, 1)] = (int32_t)item;
             return;
         }
     }
@@ -725,10 +725,8 @@ int paam_launch_lazy_safe(const paam_batch *bt, const AnalysisParams &p, int64_t
     const int64_t cap = (int64_t)per_sm * bt->ctx->n_sm;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    // every deferred system (over 16 chains or kSafeSegs segments, not narrow,
-    // outside the 32-bit bound) to the int64 kernel's list
     kern<<<(unsigned)blocks, threads, smem, stream>>>(batch_dev(bt), p, R, st, verdict, nullptr, nullptr,
-                                                      bt->list_wide, bt->counts + 1, bt->list_wide, bt->counts + 1);
+                                                      bt->list_big, bt->counts, bt->list_wide, bt->counts + 1);
     PAAM_CUDA_TRY(cudaGetLastError());
     return PAAM_OK;
 }

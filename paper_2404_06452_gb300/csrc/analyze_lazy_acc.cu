@@ -62,7 +62,8 @@ __device__ __forceinline__ uint32_t cterm(uint32_t mu, uint32_t c)
 template <int NACC>
 __device__ void lazy_acc_system(const BatchDev &b, const AnalysisParams &p, int64_t item, LazyAccSmem<NACC> &s,
                                 int lane, unsigned gm, int64_t *__restrict__ R_out, uint8_t *__restrict__ st_out,
-                                uint8_t *__restrict__ verdict, int32_t *wide_list, int32_t *wide_count)
+                                uint8_t *__restrict__ verdict, int32_t *big_list, int32_t *big_count,
+                                int32_t *wide_list, int32_t *wide_count)
 {
     int64_t sys;
     int32_t cand;
@@ -74,7 +75,7 @@ __device__ void lazy_acc_system(const BatchDev &b, const AnalysisParams &p, int6
     const int64_t c0 = b.sys_chain_off[sys];
     const int n = (int)(b.sys_chain_off[sys + 1] - c0);
     if (n > kG) {
-        if (lane == 0) wide_list[atomicAdd(wide_count, 1)] = (int32_t)item;
+        if (lane == 0) big_list[atomicAdd(big_count, 1)] = (int32_t)item;
         return;
     }
     const int16_t *rank_row = p.K > 0 ? p.ranks + (sys * p.Kc + cand_of(p, sys, cand)) * p.nmax : nullptr;
@@ -482,7 +483,8 @@ __device__ void lazy_acc_system(const BatchDev &b, const AnalysisParams &p, int6
 template <int NACC>
 __global__ void __launch_bounds__(256, NACC <= 3 ? 4 : 2) analyze_lazy_acc_kernel(BatchDev b, AnalysisParams p,
                                                                                 int64_t *R, uint8_t *st,
-                                                                                uint8_t *verdict, int32_t *wide_list,
+                                                                                uint8_t *verdict, int32_t *big_list,
+                                                                                int32_t *big_count, int32_t *wide_list,
                                                                                 int32_t *wide_count)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -493,7 +495,7 @@ __global__ void __launch_bounds__(256, NACC <= 3 ? 4 : 2) analyze_lazy_acc_kerne
     const unsigned gm = rgroup_mask<kG>();
     const int64_t n_items = p.K > 0 ? b.n_sys * p.K : b.n_sys;
     for_each_item<kG>(p, n_items, grp, groups, lane, gm, [&](int64_t i) {
-        lazy_acc_system<NACC>(b, p, i, s, lane, gm, R, st, verdict, wide_list, wide_count);
+        lazy_acc_system<NACC>(b, p, i, s, lane, gm, R, st, verdict, big_list, big_count, wide_list, wide_count);
     });
 }
 
@@ -513,7 +515,8 @@ int launch_lazy_acc_n(const paam_batch *bt, const AnalysisParams &p, int64_t *R,
     const int64_t cap = (int64_t)per_sm * bt->ctx->n_sm;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    kern<<<(unsigned)blocks, threads, smem, stream>>>(batch_dev(bt), p, R, st, verdict, bt->list_wide, bt->counts + 1);
+    kern<<<(unsigned)blocks, threads, smem, stream>>>(batch_dev(bt), p, R, st, verdict, bt->list_big, bt->counts,
+                                                      bt->list_wide, bt->counts + 1);
     PAAM_CUDA_TRY(cudaGetLastError());
     return PAAM_OK;
 }

@@ -179,6 +179,9 @@ __device__ __forceinline__ void range_per_chain(const ValidateArgs &a, int64_t s
 {
     const BatchDev &b = a.b;
     const int64_t c0 = b.sys_chain_off[s], c1 = b.sys_chain_off[s + 1];
+    if (lane == 0 && c1 > c0)
+        raise_max(&a.stats[ST_SEGMAX],
+                  (unsigned long long)(b.cb_seg_off[b.chain_cb_off[c1]] - b.cb_seg_off[b.chain_cb_off[c0]]));
     float Cmax = 0.0f, Mmax = 0.0f, dsegs = 0.0f, Dmax = 0.0f, Tmin = 3e38f;
     for (int64_t c = c0 + lane; c < c1; c += G) {
         const int64_t cb0 = b.chain_cb_off[c], cb1 = b.chain_cb_off[c + 1];
@@ -392,6 +395,7 @@ __global__ void __launch_bounds__(kValThreads, kValBlocks) validate_kernel(const
     v[ST_ECMAX] = ecmax;
     v[ST_SCMAX] = scmax;
     v[ST_DELTAMAX] = dlmax;
+    v[ST_SEGMAX] = dlmax;
     v[ST_ACCMAX] = accmax;
     v[ST_COUNT] = (unsigned long long)nmax;
     v[ST_COUNT + 1] = (unsigned long long)xmax;

@@ -137,7 +137,8 @@ __device__ __forceinline__ bool cand_pruned(const AnalysisParams &p, int64_t sys
 
 // Batch-wide maxima recorded by validation; they decide which kernels an
 // analysis needs (the 32-bit fast path covers every system when they fit).
-enum { ST_TMAX = 0, ST_DMAX, ST_ECMAX, ST_SCMAX, ST_DELTAMAX, ST_ACCMAX, ST_COUNT };
+// ST_SEGMAX: the segments of one system.
+enum { ST_TMAX = 0, ST_DMAX, ST_ECMAX, ST_SCMAX, ST_DELTAMAX, ST_ACCMAX, ST_SEGMAX, ST_COUNT };
 
 // Streams, events and page-locked words of the pipelined host analysis
 // (host_pipeline.cu), created on first use and kept for the context's life.
@@ -350,9 +351,9 @@ int paam_launch_validate_rest(const paam_batch *b, int32_t *err, unsigned long l
 
 // The lazy register-table analysis for batches with several accelerators
 // (analyze_lazy_acc.cu): 16 lanes per system, one chain per lane, instantiated
-// for the batch's accelerator count (2-4); systems over 16 chains, outside the
-// 32-bit bound or not narrow go to b->list_wide (count b->counts[1]) for the
-// int64 kernel.
+// for the batch's accelerator count (2-4); systems over 16 chains go to
+// b->list_big (count b->counts[0]), others outside the 32-bit bound or not narrow
+// to b->list_wide (count b->counts[1]) for the int64 kernel.
 int paam_launch_lazy_acc(const paam_batch *bt, const AnalysisParams &p, int64_t *R, uint8_t *st, uint8_t *verdict,
                          int64_t max_items, cudaStream_t stream);
 
@@ -362,10 +363,20 @@ int paam_launch_lazy_acc(const paam_batch *bt, const AnalysisParams &p, int64_t 
 constexpr int64_t kRecChains = (int64_t)1 << 22;
 
 // The safe reading of Lemma 4 (blocking_mode 1) in the lazy kernel (analyze_lazy.cu):
-// systems of up to 16 chains and 128 segments inside the narrow 32-bit bound, one
-// accelerator; the others are appended to b->list_wide (count b->counts[1]).
+// systems of up to 16 chains and kSafeSegs segments inside the narrow 32-bit bound,
+// one accelerator; those outside the 32-bit bound are appended to b->list_wide
+// (count b->counts[1]), the others to b->list_big (count b->counts[0]).
+constexpr int kSafeSegs = 128;
 int paam_launch_lazy_safe(const paam_batch *bt, const AnalysisParams &p, int64_t *R, uint8_t *st, uint8_t *verdict,
                           int64_t max_items, cudaStream_t stream);
+
+// The systems of b->list_big under either option (analyze_lazy_big.cu): cpl = 1, up
+// to 32 chains; cpl = 2, 33 to 64; what they cannot take goes to b->list_wide
+// (deadlines at or above kLazyDeferWideD, or more than kBigSegs segments under the
+// safe reading, among it).
+constexpr int kBigSegs = 512;
+int paam_launch_lazy_big(const paam_batch *bt, int cpl, const AnalysisParams &p, int64_t *R, uint8_t *st,
+                         uint8_t *verdict, int64_t max_items, cudaStream_t stream);
 
 // Exact int64 kernel (analyze_wide.cu) over list[0 .. *count) or, with
 // list == nullptr, over every system.

@@ -21,7 +21,9 @@ constexpr int kMaxDevices = 64;
 // [2M, 2M + 2) their counts, [2M + 4, 2M + 8) validation words,
 // [2M + 8, 2M + 8 + 2 * ST_COUNT) batch maxima (64-bit, 8-byte aligned)
 constexpr int kM = PAAM_NOALLOC_MAX_SYS;
-constexpr int kWords = 2 * kM + 8 + 2 * ST_COUNT + 6 + 6; // ... + three 64-bit work-queue counters
+constexpr int kQueueWord = 2 * kM + 8 + 2 * ST_COUNT + 2; // three 64-bit work-queue counters
+constexpr int kWords = 2 * kM + 32;
+static_assert(kQueueWord % 2 == 0 && kQueueWord + 6 <= kWords, "the counters lie inside the array");
 
 static __device__ __align__(256) int32_t g_noalloc_scratch[kWords];
 static_assert(sizeof(g_noalloc_scratch) == (size_t)PAAM_NOALLOC_MAX_SYS * 8 + 128,
@@ -114,7 +116,7 @@ extern "C" int paam_rta_analyze_noalloc(const paam_systems_view *v, const paam_a
     b.list_big = scratch;
     b.list_wide = scratch + kM;
     b.counts = scratch + 2 * kM;
-    b.queue = (unsigned long long *)(scratch + 2 * kM + 8 + 2 * ST_COUNT + 6);
+    b.queue = (unsigned long long *)(scratch + kQueueWord);
     int32_t *err = scratch + 2 * kM + 4;
     unsigned long long *stats = (unsigned long long *)(scratch + 2 * kM + 8);
 
