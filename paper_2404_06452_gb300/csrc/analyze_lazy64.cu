@@ -148,6 +148,10 @@ __device__ __forceinline__ uint32_t pair_sum(uint32_t t, const uint32_t (&tm2)[2
     return __reduce_add_sync(kFull, v);
 }
 
+// CAND: the candidate mode, an instantiation of its own so that the analysis keeps
+// its registers (with the rejection below in one kernel for both, the 1M uneven
+// systems' analysis took 1% longer).
+template <bool CAND>
 __device__ void lazy64_system(const BatchDev &b, const AnalysisParams &p, int64_t item, Lazy64Smem &s, int lane,
                               int64_t *__restrict__ R_out, uint8_t *__restrict__ st_out,
                               uint8_t *__restrict__ verdict, int32_t *wide_list, int32_t *wide_count)
@@ -155,7 +159,7 @@ __device__ void lazy64_system(const BatchDev &b, const AnalysisParams &p, int64_
     int64_t sys;
     int32_t cand;
     item_of(p, item, sys, cand);
-    if (p.K > 0 && p.early) { // candidate above the best schedulable one found so far
+    if (CAND && p.early) { // candidate above the best schedulable one found so far
         const int pruned = __shfl_sync(kFull, cand_pruned(p, sys, cand) ? 1 : 0, 0);
         if (pruned) return;
     }
@@ -166,8 +170,8 @@ __device__ void lazy64_system(const BatchDev &b, const AnalysisParams &p, int64_
         if (lane == 0) wide_list[atomicAdd(wide_count, 1)] = (int32_t)item;
         return;
     }
-    const int16_t *rank_row = p.K > 0 ? p.ranks + (sys * p.Kc + cand_of(p, sys, cand)) * p.nmax : nullptr;
-    const int32_t *xprio = p.K > 0 ? nullptr : b.exec_prio; // candidates: criticality-as-priority
+    const int16_t *rank_row = CAND ? p.ranks + (sys * p.Kc + cand_of(p, sys, cand)) * p.nmax : nullptr;
+    const int32_t *xprio = CAND ? nullptr : b.exec_prio; // candidates: criticality-as-priority
     const int64_t x0 = b.sys_exec_off[sys];
     const uint64_t kappa2 = 2 * (uint64_t)p.kappa, eps = (uint64_t)p.eps;
     const int64_t seg_base = n > 0 ? b.cb_seg_off[b.chain_cb_off[c0]] : 0;
@@ -434,7 +438,7 @@ __device__ void lazy64_system(const BatchDev &b, const AnalysisParams &p, int64_
     }
 
     // ---- own recurrence terms ------------------------------------------------
-    if (rank_row) {
+    if constexpr (CAND) {
         // a candidate with a chain whose R is above its deadline whatever its
         // interference's arrivals (the bound of cand_eval.cuh) fails at once
         bool over = false;
@@ -623,7 +627,7 @@ __device__ void lazy64_system(const BatchDev &b, const AnalysisParams &p, int64_
 
 // BLOCKS resident blocks of 256 threads per SM (three: 80 registers, which beat two
 // blocks without spills by 3.5% on the 4M-system workload); items list[0 .. *count)
-template <int BLOCKS>
+template <int BLOCKS, bool CAND>
 __global__ void __launch_bounds__(256, BLOCKS) analyze_lazy64_kernel(BatchDev b, AnalysisParams p, int64_t *R,
                                                                      uint8_t *st, uint8_t *verdict,
                                                                      const int32_t *list, const int32_t *count,
@@ -636,7 +640,7 @@ __global__ void __launch_bounds__(256, BLOCKS) analyze_lazy64_kernel(BatchDev b,
     Lazy64Smem &s = reinterpret_cast<Lazy64Smem *>(smem_raw)[grp];
     const int64_t n_items = (int64_t)*count;
     for_each_item<kW>(p, n_items, grp, groups, lane, kFull, [&](int64_t i) {
-        lazy64_system(b, p, (int64_t)list[i], s, lane, R, st, verdict, wide_list, wide_count);
+        lazy64_system<CAND>(b, p, (int64_t)list[i], s, lane, R, st, verdict, wide_list, wide_count);
     });
 }
 
@@ -648,7 +652,7 @@ int launch_lazy64(const paam_batch *bt, const AnalysisParams &p, int64_t *R, uin
     if (!list || !count || threads % 32 != 0 || threads > 256) return PAAM_E_INVAL;
     const int groups = threads / kW;
     const size_t smem = sizeof(Lazy64Smem) * groups;
-    auto kern = analyze_lazy64_kernel<3>;
+    auto kern = p.K > 0 ? analyze_lazy64_kernel<3, true> : analyze_lazy64_kernel<3, false>;
     PAAM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     PAAM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
