@@ -437,42 +437,64 @@ __device__ void lazy64_system(const BatchDev &b, const AnalysisParams &p, int64_
         }
     }
 
-    // ---- own recurrence terms ------------------------------------------------
-    if constexpr (CAND) {
-        // a candidate with a chain whose R is above its deadline whatever its
-        // interference's arrivals (the bound of cand_eval.cuh) fails at once
-        bool over = false;
+    // ---- own recurrence terms; chains known not to be schedulable --------------
+    // (the bound of analyze_lazy.cu; a candidate with such a chain fails at once)
+    uint32_t own[2], deps[2];
+    Mask needs[2];
+    uint32_t low[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const uint64_t own64 = (uint64_t)Sv[k] + (uint64_t)dlv[k] * blk[k];
+        own[k] = own64 < (uint64_t)Dv[k] + 1 ? (uint32_t)own64 : Dv[k] + 1; // values above D act the same as D + 1
+        deps[k] = (uint32_t)((uint64_t)dlv[k] * eps);
+        needs[k] = hp[k] | (hpp[k] & spins);
+        const uint32_t f = ((uint64_t)Amn[k] + blk[k]) >= 1 ? 2u : 1u;
+        low[k] = umin(Ev[k] + (user[k] ? own[k] + deps[k] + f * sums[k] : 0u), kNarrow);
+    }
+    Mask alive = all;
+    if (!counted) {
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 2; ++k) s.ssort[lane + kW * k] = low[k]; // the scan above has read it
+        __syncwarp();
+        bool over[2];
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-            const uint64_t f = ((uint64_t)Amn[k] + blk[k]) >= 1 ? 2 : 1;
-            const uint64_t low = (uint64_t)Bv[k] + Ev[k] +
-                                 (user[k] ? (uint64_t)Sv[k] + (uint64_t)dlv[k] * blk[k] + (uint64_t)dlv[k] * eps +
-                                                f * sums[k]
-                                          : 0);
-            over |= val[k] && low > Dv[k];
+            low[k] += Bv[k];
+            for (Mask m = hp[k]; m; m &= m - 1)
+                low[k] = umin(low[k] + 2u * s.ssort[__ffsll((long long)m) - 1], 1u << 31);
+            over[k] = val[k] && low[k] > Dv[k];
         }
-        if (__any_sync(kFull, over)) {
+        Mask dead = (Mask)__ballot_sync(kFull, over[0]) | ((Mask)__ballot_sync(kFull, over[1]) << 32);
+        if (CAND && dead) {
             if (lane == 0 && p.cand_ok) p.cand_ok[sys * p.Kc + cand_of(p, sys, cand)] = 0;
             __syncwarp();
             return;
         }
+        for (;;) {
+            const Mask more = dead | (Mask)__ballot_sync(kFull, (needs[0] & dead) != 0) |
+                              ((Mask)__ballot_sync(kFull, (needs[1] & dead) != 0) << 32);
+            if (more == dead) break;
+            dead = more;
+        }
+        alive = all & ~dead;
     }
+    uint32_t st0 = 0, st1 = 0; // the positions that take a step
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        if (!val[k]) continue;
         const int j = lane + kW * k;
-        const uint64_t own = (uint64_t)Sv[k] + (uint64_t)dlv[k] * blk[k];
-        const uint64_t cap = (uint64_t)Dv[k] + 1; // values above D act the same as D + 1
-        const Mask needs = hp[k] | (hpp[k] & spins);
-        s.rel[pos[k]] = Rel64{hp[k], hpp[k], hps[k], needs};
+        if (val[k]) s.needs[j] = needs[k];
+        if (!((alive >> j) & 1)) continue;
+        if (pos[k] < 32) st0 |= 1u << pos[k];
+        else st1 |= 1u << (pos[k] - 32);
+        s.rel[pos[k]] = Rel64{hp[k], hpp[k], hps[k], needs[k]};
         s.seg0[pos[k]] = seg0[k];
-        s.needs[j] = needs;
-        s.rec[pos[k]] = make_uint4(Dv[k], Bv[k] + Ev[k], (uint32_t)(own < cap ? own : cap),
-                                   (uint32_t)((uint64_t)dlv[k] * eps));
+        s.rec[pos[k]] = make_uint4(Dv[k], Bv[k] + Ev[k], own[k], deps[k]);
         // Lemma 2's sum is at least own + lb, lb = f delta sum_h S*_h (f = 2 if A* + blk >= 1)
         const uint64_t lb = (((uint64_t)Amn[k] + blk[k]) >= 1 ? 2 : 1) * (uint64_t)dlv[k] * sums[k];
         s.seg[pos[k]] = make_uint4((uint32_t)j, lb < kNarrow ? (uint32_t)lb : kNarrow, blk[k], dlv[k]);
     }
+    const Mask steps = (Mask)__reduce_or_sync(kFull, st0) | ((Mask)__reduce_or_sync(kFull, st1) << 32);
     __syncwarp();
 
     // ---- Theorem 1 (Eq. 6), chain by chain -----------------------------------
@@ -486,7 +508,8 @@ __device__ void lazy64_system(const BatchDev &b, const AnalysisParams &p, int64_
     const uint32_t k2 = (uint32_t)kappa2;
     auto chains = [&](auto counted_tag) {
     constexpr bool CNT = decltype(counted_tag)::value;
-    for (int step = 0; step < n; ++step) {
+    for (Mask left = steps; left; left &= left - 1) {
+        const int step = __ffsll((long long)left) - 1;
         const Rel64 rl = s.rel[step];
         if (rl.needs & ~sched) { // a needed H*_h is not available (the chain is DEP)
             if (rank_row) break; // a candidate fails at its first unschedulable chain

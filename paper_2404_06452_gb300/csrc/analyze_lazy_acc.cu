@@ -307,25 +307,52 @@ __device__ void lazy_acc_system(const BatchDev &b, const AnalysisParams &p, int6
         }
     }
 
-    // ---- own recurrence terms ------------------------------------------------
-    if (val) {
-        const uint64_t cap = (uint64_t)Dv + 1; // values above D act the same as D + 1
-        const Mask needs = hp | (hpp & spins);
+    // ---- own recurrence terms; chains known not to be schedulable --------------
+    // (the bound of analyze_lazy.cu, its accelerator part summed over the accelerators)
+    uint32_t own[NACC];
+    const uint32_t deps = (uint32_t)((uint64_t)dlt * eps);
+    const Mask needs = hp | (hpp & spins);
+    uint32_t low = 0;
+#pragma unroll
+    for (int u = 0; u < NACC; ++u) {
+        const uint64_t own64 = (uint64_t)Sa[u] + (uint64_t)dla[u] * blk[u];
+        own[u] = own64 < (uint64_t)Dv + 1 ? (uint32_t)own64 : Dv + 1; // values above D act the same as D + 1
+        const uint32_t f = ((uint64_t)Amn[u] + blk[u]) >= 1 ? 2u : 1u;
+        if (dla[u]) low = umin(low + own[u] + f * sums[u], kNarrow);
+    }
+    Mask alive = all;
+    if (!counted) {
+        low = umin(Ev + low + (dlt ? deps : 0u), kNarrow);
+        __syncwarp(gm);
+        s.ssort[0][j] = low; // the scans above have read it
+        __syncwarp(gm);
+        low += Bv;
+        for (Mask m = hp; m; m &= m - 1) low = umin(low + 2u * s.ssort[0][__ffs(m) - 1], 1u << 31);
+        Mask dead = __ballot_sync(gm, val && low > Dv) >> sh;
+        for (;;) {
+            const Mask more = dead | (__ballot_sync(gm, (needs & dead) != 0) >> sh);
+            if (more == dead) break;
+            dead = more;
+        }
+        alive = all & ~dead;
+    }
+    if (val) s.needs[j] = needs;
+    if ((alive >> j) & 1) {
         s.rel[pos] = make_uint4(hp, hpp, needs, seg0);
         s.chain[pos] = (uint32_t)j;
-        s.needs[j] = needs;
-        s.rec[pos] = make_uint4(Dv, Bv + Ev, (uint32_t)((uint64_t)dlt * eps), dlt);
+        s.rec[pos] = make_uint4(Dv, Bv + Ev, deps, dlt);
 #pragma unroll
         for (int u = 0; u < NACC; ++u) {
-            const uint64_t own = (uint64_t)Sa[u] + (uint64_t)dla[u] * blk[u];
             // Lemma 2's sum over the segments on u is at least own_u + lb_u, lb_u =
             // f delta_u sum_h S*_{h,u} (f = 2 if A*_u + blk_u >= 1)
             const uint64_t lb = (((uint64_t)Amn[u] + blk[u]) >= 1 ? 2 : 1) * (uint64_t)dla[u] * sums[u];
-            s.acc[pos][u] = make_uint4((uint32_t)(own < cap ? own : cap), lb < kNarrow ? (uint32_t)lb : kNarrow,
-                                       blk[u], dla[u]);
+            s.acc[pos][u] = make_uint4(own[u], lb < kNarrow ? (uint32_t)lb : kNarrow, blk[u], dla[u]);
             s.hps[pos][u] = users[u] & higher;
         }
     }
+    // the positions that take a step (none in a candidate that has failed already)
+    const Mask steps =
+        rank_row && alive != all ? 0u : __reduce_or_sync(gm, ((alive >> j) & 1) ? 1u << pos : 0u);
     __syncwarp(gm);
 
     // ---- Theorem 1 (Eq. 6), chain by chain -----------------------------------
@@ -334,7 +361,8 @@ __device__ void lazy_acc_system(const BatchDev &b, const AnalysisParams &p, int6
     const uint32_t k2 = (uint32_t)kappa2;
     auto chains = [&](auto counted_tag) {
     constexpr bool CNT = decltype(counted_tag)::value;
-    for (int step = 0; step < n; ++step) {
+    for (Mask left = steps; left; left &= left - 1) {
+        const int step = __ffs(left) - 1;
         const uint4 rl = s.rel[step];
         if (rl.z & ~sched) { // a needed H*_h is not available (the chain is DEP)
             if (rank_row) break; // a candidate fails at its first unschedulable chain

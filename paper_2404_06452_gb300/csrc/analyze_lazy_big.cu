@@ -581,27 +581,75 @@ __device__ void big_system(const BatchDev &b, const AnalysisParams &p, int64_t i
         }
     }
 
-    // ---- own recurrence terms ------------------------------------------------
+    // ---- own recurrence terms; chains known not to be schedulable --------------
+    // (the bound of analyze_lazy.cu, its accelerator part summed over the
+    // accelerators; not under the safe reading, whose blocking mostly decides)
+    uint32_t own[CPL][NACC];
+    Mask needs[CPL];
+    uint32_t low[CPL];
+    bool dead_[CPL];
 #pragma unroll
     for (int k = 0; k < CPL; ++k) {
-        if (!val[k]) continue;
+        needs[k] = hp[k] | (hpp[k] & spins);
+        low[k] = 0;
+#pragma unroll
+        for (int u = 0; u < NACC; ++u) {
+            const uint64_t own64 = (uint64_t)Sa[k][u] + (uint64_t)dla[k][u] * blk[k][u];
+            own[k][u] = own64 < (uint64_t)Dv[k] + 1 ? (uint32_t)own64 : Dv[k] + 1; // above D: as D + 1
+            const uint32_t f = ((uint64_t)Amn[k][u] + blk[k][u]) >= 1 ? 2u : 1u;
+            if (dla[k][u]) low[k] = umin(low[k] + own[k][u] + f * sums[k][u], kNarrow);
+        }
+        low[k] = umin(Ev[k] + low[k] + (uint32_t)((uint64_t)dlt[k] * eps), kNarrow);
+    }
+    Mask alive = all;
+    if (!SAFE && !counted) {
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) s.ssort[0][lane + 32 * k] = low[k]; // the scans above have read it
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) {
+            low[k] += Bv[k];
+            for (Mask m = hp[k]; m; m &= m - 1) low[k] = umin(low[k] + 2u * s.ssort[0][rlowest(m)], 1u << 31);
+            dead_[k] = val[k] && low[k] > Dv[k];
+        }
+        Mask dead = ballot_slots<CPL>(dead_);
+        for (;;) {
+#pragma unroll
+            for (int k = 0; k < CPL; ++k) dead_[k] = (needs[k] & dead) != 0;
+            const Mask more = dead | ballot_slots<CPL>(dead_);
+            if (more == dead) break;
+            dead = more;
+        }
+        alive = all & ~dead;
+    }
+    Mask steps = 0; // the positions that take a step (none in a candidate that has failed already)
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) {
         const int j = lane + 32 * k, at = pos[k];
-        const uint64_t cap = (uint64_t)Dv[k] + 1; // values above D act the same as D + 1
+        if (val[k]) s.needs[j] = needs[k];
+        if (!((alive >> j) & 1)) continue;
+        steps |= (Mask)1 << at;
         s.hp[at] = hp[k];
         s.hpp[at] = hpp[k];
-        s.needs[j] = hp[k] | (hpp[k] & spins);
         s.at[at] = make_uint2((uint32_t)j, seg0[k]);
         s.rec[at] = make_uint4(Dv[k], Bv[k] + Ev[k], (uint32_t)((uint64_t)dlt[k] * eps), dlt[k]);
 #pragma unroll
         for (int u = 0; u < NACC; ++u) {
-            const uint64_t own = (uint64_t)Sa[k][u] + (uint64_t)dla[k][u] * blk[k][u];
             // Lemma 2's sum over the segments on u is at least own_u + lb_u, lb_u =
             // f delta_u sum_h S*_{h,u} (f = 2 if A*_u + blk_u >= 1)
             const uint64_t lb = (((uint64_t)Amn[k][u] + blk[k][u]) >= 1 ? 2 : 1) * (uint64_t)dla[k][u] * sums[k][u];
-            s.acc[at][u] = make_uint4((uint32_t)(own < cap ? own : cap),
-                                      SAFE ? hsum[k] : (lb < kNarrow ? (uint32_t)lb : kNarrow), blk[k][u], dla[k][u]);
+            s.acc[at][u] = make_uint4(own[k][u], SAFE ? hsum[k] : (lb < kNarrow ? (uint32_t)lb : kNarrow), blk[k][u],
+                                      dla[k][u]);
             s.hps[at][u] = users[u] & higher[k];
         }
+    }
+    {
+        uint32_t lo = __reduce_or_sync(kFull, (uint32_t)steps), hi = 0;
+        if constexpr (CPL == 2) hi = __reduce_or_sync(kFull, (uint32_t)((uint64_t)steps >> 32));
+        steps = (Mask)lo;
+        if constexpr (CPL == 2) steps |= (Mask)hi << 32;
+        if (rank_row && alive != all) steps = 0;
     }
     __syncwarp();
 
@@ -617,7 +665,8 @@ __device__ void big_system(const BatchDev &b, const AnalysisParams &p, int64_t i
     const uint32_t k2 = (uint32_t)kappa2;
     auto chains = [&](auto counted_tag) {
     constexpr bool CNT = decltype(counted_tag)::value;
-    for (int step = 0; step < n; ++step) {
+    for (Mask left = steps; left; left &= left - 1) {
+        const int step = rlowest(left);
         const uint2 at = s.at[step];
         const int c = (int)at.x;
         if (s.needs[c] & ~sched) { // a needed H*_h is not available (the chain is DEP)
@@ -627,7 +676,7 @@ __device__ void big_system(const BatchDev &b, const AnalysisParams &p, int64_t i
         const uint4 rc = s.rec[step];
         const uint32_t D32 = rc.x, base = rc.y, deps = rc.z, dl = rc.w;
         const Mask hpc = s.hp[step], hppc = s.hpp[step];
-        uint32_t cc[CPL], ac[NACC][CPL], own[NACC], lb[NACC], Hs[NACC];
+        uint32_t cc[CPL], ac[NACC][CPL], ow[NACC], lb[NACC], Hs[NACC];
 #pragma unroll
         for (int k = 0; k < CPL; ++k) {
             const int j = lane + 32 * k;
@@ -639,14 +688,14 @@ __device__ void big_system(const BatchDev &b, const AnalysisParams &p, int64_t i
         for (int u = 0; u < NACC; ++u) {
             const uint4 ar = s.acc[step][u];
             const Mask hs_u = s.hps[step][u];
-            own[u] = ar.x;
+            ow[u] = ar.x;
             lb[u] = ar.w && !SAFE ? ar.y : kInfR; // kInfR: u unused by the chain, or its fixed points taken
             Hs[u] = ar.w && SAFE ? ar.y : kInfR;
             capped |= SAFE && ar.w && ar.y == kCapR; // a segment recurrence was cut short
 #pragma unroll
             for (int k = 0; k < CPL; ++k) ac[u][k] = ((hs_u >> (lane + 32 * k)) & 1) ? Sa[k][u] : 0u;
             uses |= ar.w ? 1u << u : 0u;
-            if (ar.w) h0 += own[u]; // Lemma 2's sum on u is never below own_u
+            if (ar.w) h0 += ow[u]; // Lemma 2's sum on u is never below own_u
         }
         const bool cpu = (hpc | hppc) != 0; // the same in every lane
         // start: B + E + H* with the interference parts of Eq. 4 empty
@@ -668,7 +717,7 @@ __device__ void big_system(const BatchDev &b, const AnalysisParams &p, int64_t i
                         if (!((uses >> u) & 1)) continue; // the same in every lane
                         const uint32_t as = slots_sum<CPL>(mu, ac[u]);
                         if (as > lb[u] && need < 0) need = u;
-                        hs += umin(Hs[u], own[u] + as); // min(Eq. 3, Eq. 4) on u, summed (R1)
+                        hs += umin(Hs[u], ow[u] + as); // min(Eq. 3, Eq. 4) on u, summed (R1)
                     }
                     if (need >= 0) { // this evaluation is taken again once that sum is known
                         if (CNT) --ev;
@@ -693,7 +742,7 @@ __device__ void big_system(const BatchDev &b, const AnalysisParams &p, int64_t i
                     uint32_t mu[CPL];
 #pragma unroll
                     for (int k = 0; k < CPL; ++k) mu[k] = rarrivals(D32, tm2[k], mg[k], lg[k]);
-                    const uint32_t lim = umin(own[u] + slots_sum<CPL>(mu, ac[u]), D32 + 1);
+                    const uint32_t lim = umin(ow[u] + slots_sum<CPL>(mu, ac[u]), D32 + 1);
                     const uint32_t blkc = s.acc[step][u].z;
                     const int64_t qb = seg_base + at.y;
                     uint32_t H32 = 0;
