@@ -14,8 +14,10 @@
 // (E: CPU WCET sum, S*: sum of A + 2 kappa, M*: largest A + 2 kappa, B: the
 // Lemma 4 blocking term, blk: the same-bucket accelerator blocking term;
 // hp, hpp, hps as in Theorem 1 and Eq. 3.)  Each value is clipped to [0, 8]
-// and stored as bf16.  One warp computes one item.
+// and stored as bf16.
 #include <cuda_bf16.h>
+
+#include <type_traits>
 
 #include "mlp.cuh"
 
@@ -23,136 +25,202 @@ namespace {
 
 constexpr int NCH = 64, NF = 16;
 
+__device__ __forceinline__ uint32_t bf16_bits(float v)
+{
+    v = fminf(fmaxf(v, 0.0f), 8.0f);
+    return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v));
+}
+
+// Group of LG lanes per item (16 for batches of up to 16 chains, else 32), lanes
+// over chains.  Issue-bound (100,000 systems of 8-16 chains: 509 us with a warp per
+// item, a division per pair and the sums in double precision; 119 us now):
+//  - a chain's ratios are divided once and kept in shared memory, not once per
+//    pair that sums them;
+//  - who is summed is a bit set (one comparison per pair), walked in index order,
+//    so every sum adds the same values in the same order as a loop over all;
+//  - the chain's sums are 64-bit integers (double precision takes 16 cycles per
+//    warp instruction here); above 2^53, where the two differ, they are taken in
+//    double precision.
+template <int LG>
 struct FeatSmem {
-    float T[NCH], D[NCH], E[NCH], Emax[NCH], S[NCH], M[NCH];
-    int32_t prio[NCH], ep[NCH], exec[NCH], core[NCH], dl[NCH], bucket[NCH];
+    static constexpr int N = LG == 16 ? 16 : NCH;
+    float uEpS[N], uE[N], uS[N], EpS[N], Emax[N], M[N];
+    int32_t prio[N], ep[N], exec[N], core[N], bucket[N];
 };
 
+// E or S* of elements [i0, i1) (each plus `add`), and the largest
+__device__ __forceinline__ void sum_and_max(const int64_t *v, int64_t i0, int64_t i1, int64_t add, float &sum, float &top)
+{
+    uint64_t t = 0, m = 0;
+    for (int64_t i = i0; i < i1; ++i) {
+        const uint64_t x = (uint64_t)(v[i] + add);
+        t += x;
+        m = x > m ? x : m;
+    }
+    sum = (float)t;
+    top = (float)m;
+    if (t >> 53) {
+        double d = 0;
+        for (int64_t i = i0; i < i1; ++i) d += (double)v[i] + (double)add;
+        sum = (float)d;
+    }
+}
+
+template <int LG>
 __global__ void __launch_bounds__(256) features_kernel(BatchDev b, const int16_t *ranks, int32_t K, int32_t nmax,
                                                        int64_t sys0, int64_t n_items, int32_t n_buckets,
                                                        int64_t kappa, int32_t slots, __nv_bfloat16 *X,
                                                        const int32_t *sys_list)
 {
-    __shared__ FeatSmem sm[8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    FeatSmem &s = sm[warp];
-    const int64_t gw = (int64_t)blockIdx.x * 8 + warp, nw = (int64_t)gridDim.x * 8;
+    using Mask = typename std::conditional<LG == 16, uint32_t, uint64_t>::type;
+    constexpr int N = FeatSmem<LG>::N, CPL = N / LG;
+    __shared__ FeatSmem<LG> sm[256 / LG];
+    const int grp = threadIdx.x / LG, lane = threadIdx.x % LG;
+    const unsigned gm = LG == 32 ? 0xffffffffu : (0xffffu << (threadIdx.x & 16u));
+    FeatSmem<LG> &s = sm[grp];
+    const int64_t gw = (int64_t)blockIdx.x * (256 / LG) + grp, nw = (int64_t)gridDim.x * (256 / LG);
     for (int64_t item = gw; item < n_items; item += nw) {
-        const int64_t sys = sys_list ? (int64_t)sys_list[sys0 + item / K] : sys0 + item / K;
-        const int32_t cand = (int32_t)(item % K);
+        const int64_t at = item / K;
+        const int64_t sys = sys_list ? (int64_t)sys_list[sys0 + at] : sys0 + at;
+        const int32_t cand = (int32_t)(item - at * K);
         const int64_t c0 = b.sys_chain_off[sys];
         const int n = (int)(b.sys_chain_off[sys + 1] - c0);
         const int64_t x0 = b.sys_exec_off[sys];
         const int16_t *row = ranks ? ranks + (sys * K + cand) * nmax : nullptr;
-        unsigned users = 0, users_hi = 0;
-        for (int c = lane; c < n; c += 32) {
+        float T[CPL], D[CPL], E[CPL], S[CPL], Emax[CPL], M[CPL], Tmin = 3.4e38f;
+        int32_t dl[CPL];
+        bool user[CPL];
+        __syncwarp(gm);
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) {
+            const int c = lane + LG * k;
+            user[k] = false;
+            dl[k] = 0;
+            T[k] = D[k] = 1.0f;
+            E[k] = S[k] = Emax[k] = M[k] = 0.0f;
+            if (c >= n) continue;
             const int64_t g = c0 + c;
             const int x = b.exec[g];
-            s.T[c] = (float)b.T[g];
-            s.D[c] = (float)b.D[g];
+            T[k] = (float)b.T[g];
+            D[k] = (float)b.D[g];
+            Tmin = fminf(Tmin, T[k]);
             s.prio[c] = row ? (n - 1 - row[c]) : b.prio[g];
             s.exec[c] = x;
             s.core[c] = b.exec_core[x0 + x];
             s.ep[c] = (!row && b.exec_prio) ? b.exec_prio[x0 + x] : INT32_MIN;
             const int64_t cb0 = b.chain_cb_off[g], cb1 = b.chain_cb_off[g + 1];
-            double E = 0, Emax = 0, S = 0, M = 0;
-            for (int64_t cb = cb0; cb < cb1; ++cb) {
-                const double e = (double)b.E[cb];
-                E += e;
-                Emax = e > Emax ? e : Emax;
-            }
             const int64_t q0 = b.cb_seg_off[cb0], q1 = b.cb_seg_off[cb1];
-            for (int64_t q = q0; q < q1; ++q) {
-                const double a = (double)b.A[q] + 2.0 * (double)kappa;
-                S += a;
-                M = a > M ? a : M;
-            }
-            s.E[c] = (float)E;
-            s.Emax[c] = (float)Emax;
-            s.S[c] = (float)S;
-            s.M[c] = (float)M;
-            s.dl[c] = (int32_t)(q1 - q0);
-            if (q1 > q0) {
-                if (c < 32) users |= 1u << c;
-                else users_hi |= 1u << (c - 32);
+            sum_and_max(b.E, cb0, cb1, 0, E[k], Emax[k]);
+            sum_and_max(b.A, q0, q1, 2 * kappa, S[k], M[k]);
+            dl[k] = (int32_t)(q1 - q0);
+            user[k] = q1 > q0;
+            s.uEpS[c] = (E[k] + S[k]) / T[k];
+            s.uE[c] = E[k] / T[k];
+            s.uS[c] = S[k] / T[k];
+            s.EpS[c] = E[k] + S[k];
+            s.Emax[c] = Emax[k];
+            s.M[c] = M[k];
+        }
+        Mask users = 0;
+#pragma unroll
+        for (int k = 0; k < CPL; ++k)
+            users |= (Mask)(__ballot_sync(gm, user[k]) >> (LG == 16 ? (threadIdx.x & 16u) : 0u)) << (LG * k);
+        const int n_users = LG == 16 ? __popc((uint32_t)users) : __popcll(users);
+        for (int off = LG / 2; off > 0; off >>= 1) Tmin = fminf(Tmin, __shfl_xor_sync(gm, Tmin, off));
+        __syncwarp(gm);
+        // relations: chains of higher priority, of the same executor, of the same core
+        Mask higher[CPL], samex[CPL], samek[CPL];
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) higher[k] = samex[k] = samek[k] = 0;
+        for (int h = 0; h < n; ++h) {
+            const int32_t ph = s.prio[h], xh = s.exec[h], kh = s.core[h];
+            const Mask bit = (Mask)1 << h;
+#pragma unroll
+            for (int k = 0; k < CPL; ++k) {
+                const int c = lane + LG * k;
+                if (c >= n) continue;
+                higher[k] |= ph > s.prio[c] ? bit : 0;
+                samex[k] |= xh == s.exec[c] ? bit : 0;
+                samek[k] |= kh == s.core[c] ? bit : 0;
             }
         }
-        users = __reduce_or_sync(0xffffffffu, users);
-        users_hi = __reduce_or_sync(0xffffffffu, users_hi);
-        const int n_users = __popc(users) + __popc(users_hi);
-        __syncwarp();
-        if (row || !b.exec_prio) // criticality-as-priority
-            for (int c = lane; c < n; c += 32) {
+        auto low_bit = [](Mask m) { return LG == 16 ? __ffs((int)(uint32_t)m) - 1 : __ffsll((long long)m) - 1; };
+        auto count = [](Mask m) { return LG == 16 ? __popc((uint32_t)m) : __popcll((uint64_t)m); };
+        if (row || !b.exec_prio) { // criticality-as-priority
+#pragma unroll
+            for (int k = 0; k < CPL; ++k) {
+                const int c = lane + LG * k;
+                if (c >= n) continue;
                 int32_t best = INT32_MIN;
-                for (int k = 0; k < n; ++k)
-                    if (s.exec[k] == s.exec[c] && s.prio[k] > best) best = s.prio[k];
+                for (Mask m = samex[k]; m; m &= m - 1) best = max(best, s.prio[low_bit(m)]);
                 s.ep[c] = best;
             }
-        float Tmin = 3.4e38f;
-        for (int c = lane; c < n; c += 32) Tmin = fminf(Tmin, s.T[c]);
-        for (int off = 16; off > 0; off >>= 1) Tmin = fminf(Tmin, __shfl_xor_sync(0xffffffffu, Tmin, off));
-        __syncwarp();
-        for (int c = lane; c < n; c += 32) { // bucket: rank among accelerator users (R2)
-            int r = 0;
-            for (int k = 0; k < n; ++k) r += (s.dl[k] > 0 && s.prio[k] > s.prio[c]) ? 1 : 0;
-            s.bucket[c] = s.dl[c] > 0 ? (int32_t)((int64_t)r * n_buckets / n_users) : -1;
         }
-        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) { // bucket: rank among accelerator users (R2)
+            const int c = lane + LG * k;
+            if (c < n)
+                s.bucket[c] =
+                    user[k] ? (int32_t)((int64_t)count(higher[k] & users) * n_buckets / n_users) : -1;
+        }
+        __syncwarp(gm);
         __nv_bfloat16 *out = X + item * (int64_t)(slots * NF);
-        for (int c = lane; c < slots; c += 32) {
-            float f[NF];
-#pragma unroll
-            for (int i = 0; i < NF; ++i) f[i] = 0.0f;
-            if (c < n) {
-                const float T = s.T[c], D = s.D[c], E = s.E[c], S = s.S[c];
-                const int32_t pc = s.prio[c], xc = s.exec[c], kc = s.core[c], ec = s.ep[c], bc = s.bucket[c];
-                int rank = 0;
-                float hp_u = 0, hpp_u = 0, hps_u = 0, hpx_d = 0, B = 0, blk = 0;
-                for (int h = 0; h < n; ++h) {
-                    if (h == c) continue;
-                    const bool hi = s.prio[h] > pc;
-                    rank += hi ? 1 : 0;
-                    if (s.exec[h] == xc) {
-                        if (hi) {
-                            hp_u += (s.E[h] + s.S[h]) / s.T[h];
-                            hpx_d += s.E[h] + s.S[h];
-                        } else {
-                            B = fmaxf(B, s.Emax[h]);
-                        }
-                    } else if (s.core[h] == kc && s.ep[h] > ec) {
-                        hpp_u += s.E[h] / s.T[h];
-                        hpx_d += s.E[h] + s.S[h];
-                    }
-                    if (s.dl[h] > 0 && hi) hps_u += s.S[h] / s.T[h];
-                    if (bc >= 0 && s.dl[h] > 0 && !hi && s.bucket[h] == bc) blk = fmaxf(blk, s.M[h]);
-                }
-                f[0] = E / T;
-                f[1] = S / T;
-                f[2] = D / T;
-                f[3] = log2f(T / Tmin) * 0.25f;
-                f[4] = (float)rank / (float)n;
-                f[5] = (float)min(s.dl[c], 16) * (1.0f / 16.0f);
-                f[6] = s.Emax[c] / D;
-                f[7] = s.M[c] / D;
-                f[8] = hp_u;
-                f[9] = hpp_u;
-                f[10] = hps_u;
-                f[11] = B / D;
-                f[12] = blk / D;
-                f[13] = (E + S) / D;
-                f[14] = hpx_d / D;
-                f[15] = 1.0f;
-#pragma unroll
-                for (int i = 0; i < NF; ++i) f[i] = fminf(fmaxf(f[i], 0.0f), 8.0f);
-            }
-            __nv_bfloat16 v[NF];
-#pragma unroll
-            for (int i = 0; i < NF; ++i) v[i] = __float2bfloat16_rn(f[i]);
+        for (int c = n + lane; c < slots; c += LG) {
             uint4 *o = (uint4 *)(out + c * NF);
-            o[0] = ((const uint4 *)v)[0];
-            o[1] = ((const uint4 *)v)[1];
+            o[0] = o[1] = make_uint4(0, 0, 0, 0);
         }
-        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) {
+            const int c = lane + LG * k;
+            if (c >= n) continue;
+            const Mask self = (Mask)1 << c;
+            const Mask hp = samex[k] & higher[k];
+            float hp_u = 0, hpp_u = 0, hps_u = 0, hpx_d = 0, B = 0, blk = 0;
+            const int32_t ec = s.ep[c];
+            Mask hpp = 0; // the same core's other executors of higher priority
+            for (Mask m = samek[k] & ~samex[k]; m; m &= m - 1) {
+                const int h = low_bit(m);
+                if (s.ep[h] > ec) hpp |= (Mask)1 << h;
+            }
+            for (Mask m = hp | hpp; m; m &= m - 1) { // in index order: hpx_d adds both
+                const int h = low_bit(m);
+                if ((hp >> h) & 1) hp_u += s.uEpS[h];
+                else hpp_u += s.uE[h];
+                hpx_d += s.EpS[h];
+            }
+            for (Mask m = samex[k] & ~higher[k] & ~self; m; m &= m - 1) B = fmaxf(B, s.Emax[low_bit(m)]);
+            for (Mask m = higher[k] & users; m; m &= m - 1) hps_u += s.uS[low_bit(m)];
+            if (user[k]) {
+                const int32_t bc = s.bucket[c];
+                for (Mask m = users & ~higher[k] & ~self; m; m &= m - 1) {
+                    const int h = low_bit(m);
+                    if (s.bucket[h] == bc) blk = fmaxf(blk, s.M[h]);
+                }
+            }
+            float f[NF];
+            f[0] = s.uE[c];
+            f[1] = s.uS[c];
+            f[2] = D[k] / T[k];
+            f[3] = log2f(T[k] / Tmin) * 0.25f;
+            f[4] = (float)count(higher[k]) / (float)n;
+            f[5] = (float)min(dl[k], 16) * (1.0f / 16.0f);
+            f[6] = Emax[k] / D[k];
+            f[7] = M[k] / D[k];
+            f[8] = hp_u;
+            f[9] = hpp_u;
+            f[10] = hps_u;
+            f[11] = B / D[k];
+            f[12] = blk / D[k];
+            f[13] = (E[k] + S[k]) / D[k];
+            f[14] = hpx_d / D[k];
+            f[15] = 1.0f;
+            uint32_t w[NF / 2];
+#pragma unroll
+            for (int i = 0; i < NF / 2; ++i) w[i] = bf16_bits(f[2 * i]) | bf16_bits(f[2 * i + 1]) << 16;
+            uint4 *o = (uint4 *)(out + c * NF);
+            o[0] = make_uint4(w[0], w[1], w[2], w[3]);
+            o[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        }
     }
 }
 
@@ -189,12 +257,6 @@ struct CandSmem {
     uint8_t ord[CF_THREADS / 16][16]; // per 16-lane segment: chain at position k
     uint8_t ord_hi[CF_THREADS / 32][16]; // positions 16..31 of 32-lane segments
 };
-
-__device__ __forceinline__ uint32_t bf16_bits(float v)
-{
-    v = fminf(fmaxf(v, 0.0f), 8.0f);
-    return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v));
-}
 
 template <int L>
 __global__ void __launch_bounds__(CF_THREADS) cand_features_kernel(BatchDev b, const int16_t *ranks, int32_t K,
@@ -453,10 +515,13 @@ int paam_launch_features(const paam_batch *b, const int16_t *ranks, int32_t K, i
             cand_features_kernel<32><<<(unsigned)blocks, CF_THREADS, 0, stream>>>(
                 batch_dev(b), ranks, K, nmax, sys0, n_systems, n_buckets, kappa, slots, X, sys_list);
     } else {
-        int64_t blocks = (n_items + 7) / 8;
+        const bool l16 = b->max_chains <= 16;
+        const int64_t per = l16 ? 16 : 8; // items per block
+        int64_t blocks = (n_items + per - 1) / per;
         if (blocks > 32 * (int64_t)b->ctx->n_sm) blocks = 32 * (int64_t)b->ctx->n_sm;
-        features_kernel<<<(unsigned)blocks, 256, 0, stream>>>(batch_dev(b), ranks, K, nmax, sys0, n_items,
-                                                              n_buckets, kappa, slots, X, sys_list);
+        auto kern = l16 ? features_kernel<16> : features_kernel<32>;
+        kern<<<(unsigned)blocks, 256, 0, stream>>>(batch_dev(b), ranks, K, nmax, sys0, n_items, n_buckets, kappa, slots,
+                                                   X, sys_list);
     }
     PAAM_CUDA_TRY(cudaGetLastError());
     paam_count_launch();

@@ -42,21 +42,38 @@ size_t n_params()
     return n;
 }
 
-// ---- labels: clip(R / D, 0, 2) for schedulable chains, 2 otherwise, -1 for padding
+// ---- labels: clip(R / D, 0, 2) for schedulable chains, 2 otherwise, -1 for padding.
+// R / D rounded once to single precision, without double precision (whose divide
+// alone bound this kernel: 72 us for 100,000 systems, 39 us now): with q near 2^24 R / D
+// the remainder 2^24 R - q D is exact in 64 bits for R < 2^38, and q plus the
+// remainder over D, both small floats, is added once.  Four slots per thread.
+__device__ __forceinline__ float ratio_of(int64_t R, int64_t D)
+{
+    if (R >> 38 || D >> 38) return (float)((double)R / (double)D);
+    const float d = (float)D;
+    const float q = rintf((float)R / d * 0x1p24f); // R <= D: at most 2^24 + 4, exact
+    const float rest = (float)((R << 24) - (int64_t)q * D) / d;
+    return fmaf(rest, 0x1p-24f, q * 0x1p-24f);
+}
+
 __global__ void labels_kernel(BatchDev b, const int64_t *R, const uint8_t *status, float *L)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < b.n_sys * NCH; i += stride) {
-        const int64_t sys = i / NCH;
-        const int c = (int)(i % NCH);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < b.n_sys * (NCH / 4); i += stride) {
+        const int64_t sys = i / (NCH / 4);
+        const int c = 4 * (int)(i % (NCH / 4));
         const int64_t c0 = b.sys_chain_off[sys];
         const int n = (int)(b.sys_chain_off[sys + 1] - c0);
-        float y = -1.0f;
-        if (c < n) {
-            const int64_t g = c0 + c;
-            y = status[g] == PAAM_ST_SCHED ? fminf((float)((double)R[g] / (double)b.D[g]), 2.0f) : 2.0f;
+        float y[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            y[k] = -1.0f;
+            if (c + k < n) {
+                const int64_t g = c0 + c + k;
+                y[k] = status[g] == PAAM_ST_SCHED ? fminf(ratio_of(R[g], b.D[g]), 2.0f) : 2.0f;
+            }
         }
-        L[i] = y;
+        *reinterpret_cast<float4 *>(L + 4 * i) = make_float4(y[0], y[1], y[2], y[3]);
     }
 }
 
@@ -422,10 +439,12 @@ int refresh_bf16(paam_model *m, cudaStream_t s)
     return PAAM_OK;
 }
 
+constexpr uint64_t kGolden = 0x9E3779B97F4A7C15ULL; // splitmix64's step
+
 // splitmix64-driven uniform in [-1, 1)
-double unif_pm1(uint64_t *x)
+__host__ __device__ double unif_pm1(uint64_t *x)
 {
-    uint64_t z = (*x += 0x9E3779B97F4A7C15ULL);
+    uint64_t z = (*x += kGolden);
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
     z ^= z >> 31;
@@ -689,6 +708,37 @@ int forward(const paam_model *m, Work &w, const __nv_bfloat16 *X, int kx, bool t
     return tc_gemm(g, w.err, s);
 }
 
+// The nodes a capturing stream's next launch follows, kept and put back: work that
+// is launched in between becomes a branch of its own.  A stream that is not
+// capturing stays a plain sequence.
+struct Branches {
+    cudaStream_t s;
+    bool on = false;
+    explicit Branches(cudaStream_t stream) : s(stream)
+    {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        on = cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusActive;
+    }
+    int now(std::vector<cudaGraphNode_t> &nodes) const
+    {
+        nodes.clear();
+        if (!on) return PAAM_OK;
+        cudaStreamCaptureStatus st;
+        const cudaGraphNode_t *d = nullptr;
+        size_t n = 0;
+        PAAM_CUDA_TRY(cudaStreamGetCaptureInfo(s, &st, nullptr, nullptr, &d, nullptr, &n));
+        nodes.assign(d, d + n);
+        return PAAM_OK;
+    }
+    int follow(std::vector<cudaGraphNode_t> &nodes) const
+    {
+        if (on)
+            PAAM_CUDA_TRY(cudaStreamUpdateCaptureDependencies(s, nodes.data(), nullptr, nodes.size(),
+                                                              cudaStreamSetCaptureDependencies));
+        return PAAM_OK;
+    }
+};
+
 // The masked MSE's gradients as the backward GEMMs leave them: per layer, the
 // split-K slices of the weight gradient in w.part[l] and the transposed output
 // gradient (dY^T, dZ^T) whose row sums are the bias gradient; grad_adamw
@@ -702,7 +752,12 @@ int backward(paam_model *m, Work &w, cudaStream_t s)
     // output layer: dW4 = dY^T H3, db4 = column sums of dY, dH3 = dY W4 (then the GELU derivative)
     const __nv_bfloat16 *dT = w.dYT; // [OUT[l]][rows]
     const __nv_bfloat16 *d = w.dY;   // [rows][OUT[l]]
+    // in a captured step each weight gradient is a branch beside the input gradients,
+    // which are what the next layer waits for: the step's chain is 11 kernels, not 14
+    Branches br(s);
+    std::vector<cudaGraphNode_t> here, end, ends;
     for (int l = 3; l >= 0; --l) {
+        if (br.now(here) != PAAM_OK) return PAAM_E_CUDA;
         const __nv_bfloat16 *inT = l == 0 ? w.XbT : w.HT[l - 1];
         TcGemm g = gemm(dT, rows, OUT[l], inT, rows, IN[l], rows);
         const DwPlan dp = dw_plan(OUT[l], IN[l], rows, sm);
@@ -716,7 +771,10 @@ int backward(paam_model *m, Work &w, cudaStream_t s)
         g.bn = dp.bn;
         int rc = tc_gemm(g, w.err, s);
         if (rc != PAAM_OK) return rc;
+        if (br.now(end) != PAAM_OK) return PAAM_E_CUDA;
+        ends.insert(ends.end(), end.begin(), end.end());
         if (l == 0) break;
+        if (br.follow(here) != PAAM_OK) return PAAM_E_CUDA;
         TcGemm h = gemm(d, OUT[l], rows, m->WbT[l], OUT[l], IN[l], OUT[l]);
         h.ep.mode = TC_EPI_DGELU;
         h.ep.M = rows;
@@ -733,7 +791,7 @@ int backward(paam_model *m, Work &w, cudaStream_t s)
         dT = w.dZT[l - 1];
         d = w.dZ[l - 1];
     }
-    return PAAM_OK;
+    return br.follow(ends);
 }
 
 // o != NULL: one AdamW step on the minibatch's gradients (bias corrections
@@ -769,6 +827,61 @@ int grad_adamw(paam_model *m, const Work &w, const paam_train_opts *o, float c1,
     PAAM_CUDA_TRY(cudaGetLastError());
     paam_count_launch();
     return PAAM_OK;
+}
+
+// The minibatch order of an epoch: the Fisher-Yates shuffle of 0..n-1 that takes
+// i = n-1 down to 1 and swaps entries i and j_i, j_i = floor(u (i + 1)) with the
+// uniforms of splitmix64 from rng, then -1 up to `total`.  On the host its chain of
+// swaps took longer than the features of the same systems (0.6 ms for 100,000); its
+// outcome can be had per entry.  Before step i, entry i holds W(i): what the last
+// step that swapped with i (the smallest i' > i with j_i' = i) brought, W(i'), or i
+// if none did; and entry j_i < i likewise W(i') for the smallest i' > i with j_i' =
+// j_i, or j_i.  So step i leaves W(i') or j_i (W(i) if j_i = i) in entry i for good.
+// The steps that share a j are a list (1 entry on average, some ln n for the first
+// ones), W a walk up such lists (a few hops).  u (i + 1) is rounded once, as on the
+// host: u itself is exact.  100,000 entries: 33 us.
+__global__ void shuffle_lists_kernel(int64_t n, uint64_t rng, int32_t *j, int32_t *head, int32_t *next)
+{
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        int64_t v = 0;
+        if (i > 0) {
+            uint64_t x = rng + kGolden * (uint64_t)(n - 1 - i); // the state before step i's draw
+            v = (int64_t)((unif_pm1(&x) * 0.5 + 0.5) * (double)(i + 1));
+            if (v > i) v -= i + 1; // the product may round up to i + 1
+            next[i] = atomicExch(&head[v], (int32_t)i);
+        }
+        j[i] = (int32_t)v;
+    }
+}
+
+// the smallest i' > i in the list of the steps that swapped with entry p, or -1
+__device__ __forceinline__ int32_t later_swap(const int32_t *head, const int32_t *next, int32_t p, int32_t i)
+{
+    int32_t best = -1;
+    for (int32_t k = head[p]; k >= 0; k = next[k])
+        if (k > i && (best < 0 || k < best)) best = k;
+    return best;
+}
+
+__global__ void shuffle_kernel(int64_t n, int64_t total, const int32_t *j, const int32_t *head, const int32_t *next,
+                               int64_t *idx)
+{
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+        if (i >= n) {
+            idx[i] = -1;
+            continue;
+        }
+        const int32_t at = j[i];
+        int32_t v = later_swap(head, next, at, (int32_t)i); // rising: the walk ends
+        if (v < 0) {
+            idx[i] = at;
+            continue;
+        }
+        for (int32_t w = later_swap(head, next, v, v); w >= 0; w = later_swap(head, next, v, v)) v = w;
+        idx[i] = v;
+    }
 }
 
 // One training step: the minibatch gather (rows idx[0 .. rows)), forward,
@@ -895,7 +1008,8 @@ extern "C" int paam_surrogate_train(paam_ctx *ctx, const paam_batch *b, const in
     const int64_t steps = (n + rows - 1) / rows;
     void *data = nullptr;
     Work w;
-    if (cudaMallocAsync(&data, (size_t)n * (2 * XW + 4 * NCH) + 8 * (size_t)steps * rows + 1024, s) != cudaSuccess) {
+    if (cudaMallocAsync(&data, (size_t)n * (2 * XW + 4 * NCH + 12) + 8 * (size_t)steps * rows + 1024, s) !=
+        cudaSuccess) {
         cudaGetLastError();
         rc = PAAM_E_NOMEM;
     }
@@ -903,28 +1017,25 @@ extern "C" int paam_surrogate_train(paam_ctx *ctx, const paam_batch *b, const in
     __nv_bfloat16 *X = (__nv_bfloat16 *)data;
     float *L = (float *)((char *)data + (size_t)n * 2 * XW);
     int64_t *idx_dev = (int64_t *)((char *)L + (size_t)n * 4 * NCH);
+    int32_t *shuf_j = (int32_t *)(idx_dev + steps * rows), *shuf_head = shuf_j + n, *shuf_next = shuf_head + n;
     if (rc == PAAM_OK) rc = paam_launch_features(b, nullptr, 1, 0, 0, n, o->n_buckets, o->kappa_ns, XW, X, s);
     if (rc == PAAM_OK) {
-        labels_kernel<<<grid_for(n * NCH, 256, ctx->n_sm), 256, 0, s>>>(batch_dev(b), R, status, L);
+        labels_kernel<<<grid_for(n * (NCH / 4), 256, ctx->n_sm), 256, 0, s>>>(batch_dev(b), R, status, L);
         if (cudaGetLastError() != cudaSuccess) rc = PAAM_E_CUDA;
         paam_count_launch();
         if (cudaMemsetAsync(w.err, 0, 4, s) != cudaSuccess) rc = PAAM_E_CUDA;
     }
-    std::vector<int64_t> idx((size_t)(steps * rows));
     StepGraph sg;
     uint64_t rng = o->seed ^ 0x5DEECE66DULL ^ (uint64_t)m->step;
     for (int e = 0; e < o->epochs && rc == PAAM_OK; ++e) {
         // minibatch order: a fresh permutation of the systems, padded with -1
-        for (int64_t i = 0; i < (int64_t)idx.size(); ++i) idx[i] = i < n ? i : -1;
-        for (int64_t i = n - 1; i > 0; --i) {
-            const int64_t j = (int64_t)((unif_pm1(&rng) * 0.5 + 0.5) * (double)(i + 1)) % (i + 1);
-            const int64_t t = idx[i];
-            idx[i] = idx[j];
-            idx[j] = t;
-        }
-        if (cudaMemcpyAsync(idx_dev, idx.data(), 8 * idx.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-            cudaMemsetAsync(w.loss, 0, 4, s) != cudaSuccess)
-            rc = PAAM_E_CUDA;
+        if (cudaMemsetAsync(shuf_head, 0xff, 4 * (size_t)n, s) != cudaSuccess) rc = PAAM_E_CUDA;
+        shuffle_lists_kernel<<<grid_for(n, 256, ctx->n_sm), 256, 0, s>>>(n, rng, shuf_j, shuf_head, shuf_next);
+        shuffle_kernel<<<grid_for(steps * rows, 256, ctx->n_sm), 256, 0, s>>>(n, steps * rows, shuf_j, shuf_head,
+                                                                             shuf_next, idx_dev);
+        rng += kGolden * (uint64_t)(n > 0 ? n - 1 : 0);
+        paam_count_launch(2);
+        if (cudaGetLastError() != cudaSuccess || cudaMemsetAsync(w.loss, 0, 4, s) != cudaSuccess) rc = PAAM_E_CUDA;
         for (int64_t st = 0; st < steps && rc == PAAM_OK; ++st) {
             m->step += 1;
             const float c1 = 1.0f - powf(o->beta1, (float)m->step), c2 = 1.0f - powf(o->beta2, (float)m->step);
