@@ -185,8 +185,9 @@ void paam_batch_free(paam_batch *b);
  *                    admission test of Sec. IV-A), else 0
  * verdict may be NULL.  Results are bit-identical to the definition for any
  * launch configuration.  The first call for a given (outputs, options,
- * launch configuration) captures the analysis into a CUDA graph owned by the
- * batch; later calls with the same key replay it on `stream`.  A batch may be
+ * launch configuration) launches the analysis; the second captures it into a
+ * CUDA graph owned by the batch, and later calls with the same key replay it
+ * on `stream`.  A batch may be
  * analysed by one host thread at a time.  Errors: PAAM_E_INVAL (NULL outputs, n_buckets < 1),
  * PAAM_E_RANGE (eps or kappa above PAAM_MAX_OVERHEAD), PAAM_E_INVAL
  * (blocking_mode not 0 or 1), PAAM_E_CUDA (launch failure).

@@ -599,13 +599,15 @@ int paam_enqueue_analysis(const paam_batch *b, const AnalysisParams &p, const La
         if (n_kernels) *n_kernels = 1;
         return rc;
     }
-    PAAM_CUDA_TRY(cudaMemsetAsync(b->counts, 0, 2 * sizeof(int32_t), stream));
+    // the lists' counts and, right after them, the queue's counters
+    const bool queue = cfg.queue > 0 && b->queue;
+    PAAM_CUDA_TRY(cudaMemsetAsync(b->counts, 0, 2 * sizeof(int32_t) + (queue ? 3 * sizeof(unsigned long long) : 0),
+                                  stream));
     // per pass: its own work-queue counter, or static shares
     AnalysisParams pm = p, pb = p, pw = p;
     pm.queue_batch = pb.queue_batch = pw.queue_batch = 0;
     pm.sys_order = pb.sys_order = pw.sys_order = cfg.binned ? b->sys_order : nullptr;
-    if (cfg.queue > 0 && b->queue) {
-        PAAM_CUDA_TRY(cudaMemsetAsync(b->queue, 0, 3 * sizeof(unsigned long long), stream));
+    if (queue) {
         pm.queue = b->queue;
         pb.queue = b->queue + 1;
         pw.queue = b->queue + 2;

@@ -26,23 +26,9 @@ namespace {
 
 constexpr size_t kMinChunkBytes = (size_t)64 << 20; // input bytes of the smallest automatic chunk
 constexpr int kMaxChunks = 4096;
-constexpr size_t kWords = 4 * sizeof(int32_t) + ST_COUNT * sizeof(unsigned long long); // per chunk
+constexpr size_t kWords = sizeof(ValidateWords); // per chunk
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
-
-// validation words of every chunk: {0, INT32_MAX, 0, 0} then zeroed maxima
-__global__ void init_words(char *w, int64_t n_chunks)
-{
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n_chunks; k += (int64_t)gridDim.x * blockDim.x) {
-        int32_t *e = (int32_t *)(w + kWords * (size_t)k);
-        e[0] = 0;
-        e[1] = INT32_MAX;
-        e[2] = 0;
-        e[3] = 0;
-        unsigned long long *st = (unsigned long long *)(e + 4);
-        for (int i = 0; i < ST_COUNT; ++i) st[i] = 0;
-    }
-}
 
 // the context's streams, at least n_ev events and page-locked words of at least `bytes`
 int pipe_get(paam_ctx *ctx, int n_ev, size_t bytes, HostPipe **out)
@@ -234,7 +220,7 @@ extern "C" int paam_rta_analyze_host(paam_ctx *ctx, const paam_systems_view *v, 
     t.list_wide = (int32_t *)p;
     p += align256(list_bytes);
     t.counts = (int32_t *)p;
-    t.queue = (unsigned long long *)(t.counts + 8);
+    t.queue = (unsigned long long *)(t.counts + 2);
     p += 256;
     char *wdev = p;
     char *whost = (char *)pl->words;
@@ -244,11 +230,8 @@ extern "C" int paam_rta_analyze_host(paam_ctx *ctx, const paam_systems_view *v, 
         cudaStreamWaitEvent(pl->val, *ev_alloc, 0) != cudaSuccess ||
         cudaStreamWaitEvent(pl->out, *ev_alloc, 0) != cudaSuccess)
         rc = PAAM_E_CUDA;
-    if (rc == PAAM_OK) {
-        init_words<<<1, 256, 0, pl->val>>>(wdev, n_chunks);
-        if (cudaGetLastError() != cudaSuccess) rc = PAAM_E_CUDA;
-    }
-    unsigned launches = 1;
+    if (rc == PAAM_OK && cudaMemsetAsync(wdev, 0, kWords * (size_t)n_chunks, pl->val) != cudaSuccess) rc = PAAM_E_CUDA;
+    unsigned launches = 0;
 
     // ---- copies of every chunk (copy stream), validation of every chunk as it lands
     // (validation stream), each chunk's words back to the page-locked buffer

@@ -150,13 +150,19 @@ struct HostPipe {
     size_t words_bytes = 0;
 };
 
+// What a validation leaves, zeroed before it (one word block, so that one fill and
+// one copy back serve it): err = {code, undecided, max chains, max executors}.
+struct ValidateWords {
+    int32_t err[4];
+    unsigned long long stats[ST_COUNT];
+};
+
 struct paam_ctx {
     int device;
     int n_sm;
     int max_smem_optin;
     cudaStream_t capture_stream; // private stream used to capture analysis graphs
-    int32_t *d_err;        // validation: [0] code, [1] undecided, [2] max chains, [3] max executors
-    unsigned long long *d_stats; // validation: ST_* maxima
+    ValidateWords *d_words;
     HostPipe *pipe;
 };
 
@@ -178,13 +184,17 @@ struct paam_batch {
     // [1] systems deferred to the exact int64 kernel, both n_sys long; counts
     int32_t *list_big, *list_wide;
     int32_t *counts; // [0] big, [1] wide
-    unsigned long long *queue; // [3] work-queue counters of the three passes (NULL: none)
+    unsigned long long *queue; // [3] work-queue counters of the three passes, right after counts
     int32_t *sys_order;        // [n_sys] systems by increasing chain count within windows of consecutive systems (NULL: not built)
     void *block;
     size_t block_bytes;
     int cfg_index; // launch configuration (index into kLaunchCfgs)
-    // the analysis captured as a CUDA graph, replayed while its key matches
+    // the analysis captured as a CUDA graph at the second call with one key, replayed
+    // while the key matches (key_seen: the key holds some earlier call's values)
     cudaGraphExec_t graph;
+    bool key_seen, first_open; // first_open: the first call's launches may still run
+    cudaEvent_t first_ev;      // recorded after them on first_stream
+    cudaStream_t first_stream;
     int graph_kernels;
     struct {
         int64_t *R;
@@ -327,8 +337,7 @@ constexpr uint32_t kIterCap = (uint32_t)PAAM_MAX_ITER;
 int paam_enqueue_analysis(const paam_batch *b, const AnalysisParams &p, const LaunchCfg &cfg, int64_t *R,
                           uint8_t *status, uint8_t *verdict, cudaStream_t stream, int *n_kernels);
 
-// Validation kernel (api.cu): err = {code, undecided, max chains, max executors}
-// (initialise to {0, INT32_MAX, 0, 0}), stats = ST_* maxima (zeroed).  Once the
+// Validation kernel (api.cu): err and stats as in ValidateWords.  Once the
 // words are on the host and paam_validate_undecided says so, the batch (valid so
 // far) also takes paam_launch_validate_rest, which adds to the same words.  The
 // maxima of a chain's E, A and segments may be their system's sums (below 2^29),

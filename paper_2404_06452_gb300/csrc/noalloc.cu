@@ -17,13 +17,11 @@
 namespace {
 
 constexpr int kMaxDevices = 64;
-// layout in 32-bit words: [0, M) wide-configuration list, [M, 2M) int64 list,
-// [2M, 2M + 2) their counts, [2M + 4, 2M + 8) validation words,
-// [2M + 8, 2M + 8 + 2 * ST_COUNT) batch maxima (64-bit, 8-byte aligned)
+// layout in 32-bit words: [0, M) deferral list, [M, 2M) int64 list, [2M, 2M + 2) their
+// counts, [2M + 2, 2M + 8) three 64-bit work-queue counters, then the validation words
 constexpr int kM = PAAM_NOALLOC_MAX_SYS;
-constexpr int kQueueWord = 2 * kM + 8 + 2 * ST_COUNT + 2; // three 64-bit work-queue counters
 constexpr int kWords = 2 * kM + 32;
-static_assert(kQueueWord % 2 == 0 && kQueueWord + 6 <= kWords, "the counters lie inside the array");
+static_assert(sizeof(ValidateWords) <= 24 * sizeof(int32_t), "the validation words lie inside the array");
 
 static __device__ __align__(256) int32_t g_noalloc_scratch[kWords];
 static_assert(sizeof(g_noalloc_scratch) == (size_t)PAAM_NOALLOC_MAX_SYS * 8 + 128,
@@ -116,33 +114,27 @@ extern "C" int paam_rta_analyze_noalloc(const paam_systems_view *v, const paam_a
     b.list_big = scratch;
     b.list_wide = scratch + kM;
     b.counts = scratch + 2 * kM;
-    b.queue = (unsigned long long *)(scratch + kQueueWord);
-    int32_t *err = scratch + 2 * kM + 4;
-    unsigned long long *stats = (unsigned long long *)(scratch + 2 * kM + 8);
+    b.queue = (unsigned long long *)(b.counts + 2);
+    ValidateWords *dw = (ValidateWords *)(scratch + 2 * kM + 8);
 
     // the array keeps the previous call's contents: reset what must start at zero
-    const int32_t err0[4] = {0, 0x7fffffff, 0, 0};
-    PAAM_CUDA_TRY(cudaMemcpyAsync(err, err0, sizeof(err0), cudaMemcpyHostToDevice, stream));
-    PAAM_CUDA_TRY(cudaMemsetAsync(stats, 0, ST_COUNT * sizeof(unsigned long long), stream));
-    rc = paam_launch_validate(&b, v->acc, err, stats, stream);
+    ValidateWords words;
+    PAAM_CUDA_TRY(cudaMemsetAsync(dw, 0, sizeof(*dw), stream));
+    rc = paam_launch_validate(&b, v->acc, dw->err, dw->stats, stream);
     if (rc != PAAM_OK) return rc;
-    int32_t herr[4];
-    unsigned long long hstats[ST_COUNT];
-    PAAM_CUDA_TRY(cudaMemcpyAsync(herr, err, sizeof(herr), cudaMemcpyDeviceToHost, stream));
-    PAAM_CUDA_TRY(cudaMemcpyAsync(hstats, stats, sizeof(hstats), cudaMemcpyDeviceToHost, stream));
+    PAAM_CUDA_TRY(cudaMemcpyAsync(&words, dw, sizeof(words), cudaMemcpyDeviceToHost, stream));
     PAAM_CUDA_TRY(cudaStreamSynchronize(stream));
-    if (paam_validate_undecided(herr)) {
-        rc = paam_launch_validate_rest(&b, err, stats, stream);
+    if (paam_validate_undecided(words.err)) {
+        rc = paam_launch_validate_rest(&b, dw->err, dw->stats, stream);
         if (rc != PAAM_OK) return rc;
-        PAAM_CUDA_TRY(cudaMemcpyAsync(herr, err, sizeof(herr), cudaMemcpyDeviceToHost, stream));
-        PAAM_CUDA_TRY(cudaMemcpyAsync(hstats, stats, sizeof(hstats), cudaMemcpyDeviceToHost, stream));
+        PAAM_CUDA_TRY(cudaMemcpyAsync(&words, dw, sizeof(words), cudaMemcpyDeviceToHost, stream));
         PAAM_CUDA_TRY(cudaStreamSynchronize(stream));
     }
-    if (herr[0] != 0) return herr[0];
-    b.max_chains = herr[2];
-    b.max_exec = herr[3];
-    for (int i = 0; i < ST_COUNT; ++i) b.stats[i] = hstats[i];
-    b.acc = hstats[ST_ACCMAX] > 0 ? (int32_t *)v->acc : nullptr;
+    if (words.err[0] != 0) return words.err[0];
+    b.max_chains = words.err[2];
+    b.max_exec = words.err[3];
+    for (int i = 0; i < ST_COUNT; ++i) b.stats[i] = words.stats[i];
+    b.acc = words.stats[ST_ACCMAX] > 0 ? (int32_t *)v->acc : nullptr;
 
     AnalysisParams p = {};
     p.n_buckets = o->n_buckets;

@@ -89,8 +89,8 @@ int search_ordered_impl(paam_ctx *ctx, const paam_batch *b, const paam_analysis_
     bs.list_big = (int32_t *)tmp;
     bs.list_wide = (int32_t *)((char *)tmp + list_bytes);
     bs.counts = (int32_t *)((char *)tmp + 2 * list_bytes);
-    int32_t *err = bs.counts + 4;
-    bs.queue = (unsigned long long *)(bs.counts + 8); // bytes 32..55 of the 64-byte tail
+    bs.queue = (unsigned long long *)(bs.counts + 2);
+    int32_t *err = bs.counts + 8; // the 64-byte tail: counts, queue, error word
     bs.graph = nullptr;
 
     int rc = PAAM_OK;
