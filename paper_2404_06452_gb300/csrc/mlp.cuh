@@ -9,9 +9,8 @@
 // Epilogue applied to each fp32 accumulator tile of the tensor-core GEMM.
 enum TcEpiMode {
     TC_EPI_STORE_F32 = 0,  // C = acc (with split_stride: split z writes C + z * split_stride)
-    TC_EPI_BIAS_GELU = 1,  // Z = bf16(acc + bias); H = bf16(gelu(Z)); HT = H^T (optional)
+    TC_EPI_BIAS_GELU = 1,  // H = bf16(gelu(acc + bias))
     TC_EPI_BIAS_F32 = 2,   // C = acc + bias
-    TC_EPI_DGELU = 3,      // H = bf16(acc * gelu'(Zin)); HT = H^T (optional)
     TC_EPI_ATOMIC_F32 = 4, // C += acc (split-K partial sums)
     TC_EPI_ROWMAX = 5,     // C[row] = max(C[row], 0, max over the row's valid columns of acc + bias)
 };
@@ -21,14 +20,8 @@ struct TcEpilogue {
     float *C;
     int ldc;
     const float *bias;             // [N]
-    const __nv_bfloat16 *Zin;      // pre-activation read by TC_EPI_DGELU
-    int ldzin;
-    __nv_bfloat16 *Z;              // pre-activation written by TC_EPI_BIAS_GELU
-    int ldz;
-    __nv_bfloat16 *H;              // activation (BIAS_GELU) or input gradient (DGELU), row-major
+    __nv_bfloat16 *H;              // activation, row-major
     int ldh;
-    __nv_bfloat16 *HT;             // H transposed ([N][M]), optional
-    int ldht;
     // TC_EPI_ROWMAX: row r belongs to system sys0 + r / rows_per_sys (with
     // sys_list, to system sys_list[sys0 + r / rows_per_sys]), whose chain count
     // (sys_off[s + 1] - sys_off[s]) is the number of valid columns; C[r] must
@@ -58,9 +51,34 @@ struct TcGemm {
     int K, splits;
     TcEpilogue ep;
     int bn;
+    int mn; // 1: A is [K][a_rows] and B [K][b_rows] in memory, C = A^T B (bn 64 or 256)
 };
 
 int tc_gemm(const TcGemm &g, int32_t *err, cudaStream_t stream);
+
+// TMA map of a bf16 row-major matrix [rows][ld] of which cols columns are valid: tiles
+// of box_rows x 64 in the 128-byte swizzle, zeros outside.
+bool tc_make_map(CUtensorMap *m, const __nv_bfloat16 *base, int rows, int cols, int ld, int box_rows);
+
+// The chain of a training step over `rows` minibatch rows (a multiple of 128):
+// forward, masked mean-squared error and input gradients (mlp_train.cu).  Reads X
+// [rows][1024], the layers' bf16 weights W [out][in] and WT [in][out] and the fp32
+// labels L [rows][64] (< 0: none; *count of them valid); writes the activations H and
+// the gradients dZ [rows][256] and dY [rows][64] (and Z, its own), and
+// leaves each bias gradient as rows / 32 sums of 32 rows in bias_part ([rows / 32]
+// [kPartCols], the layers' biases one after another) and behind them the loss's, two
+// columns (one per half of the outputs).
+constexpr int kBiasCols = 3 * 256 + 64, kPartCols = kBiasCols + 32;
+struct TrainChain {
+    int rows;
+    const float *bias[4];
+    __nv_bfloat16 *Z, *H[3], *dY, *dZ[3];
+    const float *L, *count;
+    float *bias_part;
+    int32_t *err;
+};
+int paam_train_chain(const TrainChain &c, const __nv_bfloat16 *X, const __nv_bfloat16 *const (&W)[4],
+                     const __nv_bfloat16 *const (&WT)[4], cudaStream_t stream);
 
 
 

@@ -82,39 +82,15 @@ __device__ __forceinline__ void epilogue_chunk(const TcEpilogue &ep, int row, in
             if (col0 + i < ep.N) atomicAdd(c + i, a[i]);
         break;
     }
-    case TC_EPI_BIAS_GELU:
-    case TC_EPI_DGELU: {
-        __nv_bfloat16 out[32];
-        if (ep.mode == TC_EPI_BIAS_GELU) {
-            add_bias(ep, col0, full, a);
-            if (ep.Z && full) { // the pre-activation, kept for the backward pass
-                __nv_bfloat162 zb[16];
+    case TC_EPI_BIAS_GELU: {
+        __nv_bfloat162 out[16];
+        add_bias(ep, col0, full, a);
 #pragma unroll
-                for (int i = 0; i < 16; ++i) zb[i] = __floats2bfloat162_rn(a[2 * i], a[2 * i + 1]);
-                uint4 *z = (uint4 *)(ep.Z + (size_t)row * ep.ldz + col0);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) z[i] = ((const uint4 *)zb)[i];
-            }
-#pragma unroll
-            for (int i = 0; i < 16; ++i)
-                ((__nv_bfloat162 *)out)[i] = __floats2bfloat162_rn(gelu(a[2 * i]), gelu(a[2 * i + 1]));
-        } else {
-            const __nv_bfloat16 *zin = ep.Zin + (size_t)row * ep.ldzin + col0;
-            __nv_bfloat16 zb[32];
-            if (full) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) ((uint4 *)zb)[i] = ((const uint4 *)zin)[i];
-            }
-#pragma unroll
-            for (int i = 0; i < 32; ++i) out[i] = __float2bfloat16_rn(a[i] * gelu_grad(__bfloat162float(zb[i])));
-        }
+        for (int i = 0; i < 16; ++i) out[i] = __floats2bfloat162_rn(gelu(a[2 * i]), gelu(a[2 * i + 1]));
         if (full) {
             uint4 *h = (uint4 *)(ep.H + (size_t)row * ep.ldh + col0);
 #pragma unroll
             for (int i = 0; i < 4; ++i) h[i] = ((const uint4 *)out)[i];
-            if (ep.HT) // one column at a time: the warp's 32 consecutive rows are contiguous
-#pragma unroll
-                for (int i = 0; i < 32; ++i) ep.HT[(size_t)(col0 + i) * ep.ldht + row] = out[i];
         }
         break;
     }
@@ -136,7 +112,9 @@ struct GemmSmem {
 // warps per TMEM lane quadrant, one per half of the tile's columns).
 constexpr int kGemmThreads = 320;
 
-template <int BN, int STAGES>
+// MN: A is [K][M] and B [K][N] in memory (TcGemm::mn): tiles come as boxes of 64 x 64
+// and the tensor core reads them transposed, so no transposed copies are needed.
+template <int BN, int STAGES, bool MN>
 __global__ void __launch_bounds__(kGemmThreads, 2) tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
                                                       const __grid_constant__ CUtensorMap tmB, int kb_total,
                                                       int kb_per_split, TcEpilogue ep, int32_t *err)
@@ -190,12 +168,19 @@ __global__ void __launch_bounds__(kGemmThreads, 2) tc_gemm_kernel(const __grid_c
             uint8_t *a = smem + s * L::STAGE;
             uint8_t *b = a + L::A_BYTES;
             tc::mbar_expect_tx(&full[s], L::STAGE);
-            tc::tma_load_2d(a, &tmA, &full[s], (kb0 + i) * BK, m0);
-            tc::tma_load_2d(b, &tmB, &full[s], (kb0 + i) * BK, n0);
+            if constexpr (MN) { // columns past the matrix read zeros
+                for (int x = 0; x < BM / 64; ++x)
+                    tc::tma_load_2d(a + x * 8192, &tmA, &full[s], m0 + 64 * x, (kb0 + i) * BK);
+                for (int x = 0; x < BN / 64; ++x)
+                    tc::tma_load_2d(b + x * 8192, &tmB, &full[s], n0 + 64 * x, (kb0 + i) * BK);
+            } else {
+                tc::tma_load_2d(a, &tmA, &full[s], (kb0 + i) * BK, m0);
+                tc::tma_load_2d(b, &tmB, &full[s], (kb0 + i) * BK, n0);
+            }
         }
         *issued = i;
     } else if (warp == 1 && lane == 0) { // ---- MMA issuer
-        constexpr uint32_t idesc = tc::idesc_bf16(BM, BN);
+        constexpr uint32_t idesc = MN ? tc::idesc_bf16_mn(BM, BN) : tc::idesc_bf16(BM, BN);
         bool ok = nkb > 0;
         for (int i = 0; i < nkb; ++i) {
             const int s = i % STAGES, r = i / STAGES;
@@ -209,9 +194,14 @@ __global__ void __launch_bounds__(kGemmThreads, 2) tc_gemm_kernel(const __grid_c
             const uint32_t a = tc::smem_u32(smem + s * L::STAGE);
             const uint32_t b = a + L::A_BYTES;
 #pragma unroll
-            for (int j = 0; j < BK / 16; ++j) // K = 16 per instruction: step 32 bytes inside the swizzle atom
-                tc::mma_bf16(tmem, tc::desc_sw128(a + 32 * j), tc::desc_sw128(b + 32 * j), idesc,
-                             (i > 0 || j > 0) ? 1u : 0u);
+            for (int j = 0; j < BK / 16; ++j) { // K = 16 per instruction
+                if constexpr (MN) // 16 contraction rows of 128 bytes
+                    tc::mma_bf16(tmem, tc::desc_mn_sw128(a + 2048 * j), tc::desc_mn_sw128(b + 2048 * j), idesc,
+                                 (i > 0 || j > 0) ? 1u : 0u);
+                else // 32 bytes inside the swizzle atom
+                    tc::mma_bf16(tmem, tc::desc_sw128(a + 32 * j), tc::desc_sw128(b + 32 * j), idesc,
+                                 (i > 0 || j > 0) ? 1u : 0u);
+            }
             tc::mma_commit(&empty[s]); // frees the stage once these MMAs have read it
         }
         if (ok) tc::mma_commit(done);
@@ -493,8 +483,9 @@ EncodeTiledFn encode_fn()
     return fn;
 }
 
-// bf16 row-major matrix [rows][ld], tile box_rows x 64, 128-byte swizzle, zeros outside
-bool make_map(CUtensorMap *m, const __nv_bfloat16 *base, int rows, int cols, int ld, int box_rows)
+} // namespace
+
+bool tc_make_map(CUtensorMap *m, const __nv_bfloat16 *base, int rows, int cols, int ld, int box_rows)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
@@ -507,19 +498,23 @@ bool make_map(CUtensorMap *m, const __nv_bfloat16 *base, int rows, int cols, int
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN, int STAGES>
+namespace {
+
+template <int BN, int STAGES, bool MN>
 int launch_bn(const TcGemm &g, int32_t *err, cudaStream_t stream)
 {
     CUtensorMap ma, mb;
-    if (!make_map(&ma, g.A, g.a_rows, g.K, g.lda, BM) || !make_map(&mb, g.B, g.b_rows, g.K, g.ldb, BN))
+    if (MN ? (!tc_make_map(&ma, g.A, g.K, g.a_rows, g.lda, 64) || !tc_make_map(&mb, g.B, g.K, g.b_rows, g.ldb, 64))
+           : (!tc_make_map(&ma, g.A, g.a_rows, g.K, g.lda, BM) || !tc_make_map(&mb, g.B, g.b_rows, g.K, g.ldb, BN)))
         return PAAM_E_CUDA;
     const int kb_total = g.K / BK;
     const int splits = g.splits < 1 ? 1 : (g.splits > kb_total ? kb_total : g.splits);
     const int per = (kb_total + splits - 1) / splits;
     const dim3 grid((unsigned)((g.ep.M + BM - 1) / BM), (unsigned)(g.ep.N / BN), (unsigned)((kb_total + per - 1) / per));
     const int smem = GemmSmem<BN, STAGES>::TOTAL;
-    PAAM_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_kernel<BN, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    tc_gemm_kernel<BN, STAGES><<<grid, kGemmThreads, smem, stream>>>(ma, mb, kb_total, per, g.ep, err);
+    PAAM_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_kernel<BN, STAGES, MN>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    tc_gemm_kernel<BN, STAGES, MN><<<grid, kGemmThreads, smem, stream>>>(ma, mb, kb_total, per, g.ep, err);
     PAAM_CUDA_TRY(cudaGetLastError());
     paam_count_launch();
     return PAAM_OK;
@@ -528,12 +523,12 @@ int launch_bn(const TcGemm &g, int32_t *err, cudaStream_t stream)
 // Short K (at most 4 steps of 64) needs no deeper ring than 2 stages; the
 // smaller footprint lets 2 CTAs share an SM, so one CTA's epilogue overlaps
 // the other's loads and MMAs (TMEM: 2 x 256 columns at most).
-template <int BN>
+template <int BN, bool MN = false>
 int launch_bn_depth(const TcGemm &g, int32_t *err, cudaStream_t stream)
 {
     const int per = g.splits > 1 ? (g.K / BK + g.splits - 1) / g.splits : g.K / BK;
-    if (per <= 4) return launch_bn<BN, 2>(g, err, stream);
-    return launch_bn<BN, 4>(g, err, stream);
+    if (per <= 4) return launch_bn<BN, 2, MN>(g, err, stream);
+    return launch_bn<BN, 4, MN>(g, err, stream);
 }
 
 } // namespace
@@ -566,10 +561,10 @@ template <int BN>
 int launch_persistent(const TcGemm &g, int32_t *err, cudaStream_t stream)
 {
     CUtensorMap ma, mb, mh;
-    if (!make_map(&ma, g.A, g.a_rows, g.K, g.lda, BM) || !make_map(&mb, g.B, g.b_rows, g.K, g.ldb, BN))
+    if (!tc_make_map(&ma, g.A, g.a_rows, g.K, g.lda, BM) || !tc_make_map(&mb, g.B, g.b_rows, g.K, g.ldb, BN))
         return PAAM_E_CUDA;
     // the TMA-store epilogue: bias + GELU into H only, every column of the tile valid, H 16-byte aligned rows
-    int tma_out = g.ep.mode == TC_EPI_BIAS_GELU && !g.ep.Z && !g.ep.HT && g.ep.H && g.ep.bias && g.ep.N == BN &&
+    int tma_out = g.ep.mode == TC_EPI_BIAS_GELU && g.ep.H && g.ep.bias && g.ep.N == BN &&
                   g.ep.ldh % 8 == 0 && ((uintptr_t)g.ep.H & 15) == 0;
     if (tma_out && !make_store_map(&mh, g.ep.H, g.ep.M, g.ep.N, g.ep.ldh)) tma_out = 0;
     if (!tma_out) mh = ma; // unused
@@ -592,6 +587,11 @@ int tc_gemm(const TcGemm &g, int32_t *err, cudaStream_t stream)
         return PAAM_E_INVAL;
     if (g.ep.split_stride && (g.ep.mode != TC_EPI_STORE_F32 || g.splits < 1)) return PAAM_E_INVAL;
     if (g.bn && ((g.bn != 64 && g.bn != 128 && g.bn != 256) || g.ep.N % g.bn)) return PAAM_E_INVAL;
+    if (g.mn) { // the weight gradients: 64 or 256 columns
+        if (g.bn == 64) return launch_bn_depth<64, true>(g, err, stream);
+        if (g.bn == 256) return launch_bn_depth<256, true>(g, err, stream);
+        return PAAM_E_INVAL;
+    }
     if (g.bn == 64) return launch_bn_depth<64>(g, err, stream);
     if (g.bn == 128) return launch_bn_depth<128>(g, err, stream);
     // one column tile, short K, many row tiles: weights stay resident, epilogue overlaps MMA

@@ -77,139 +77,60 @@ __global__ void labels_kernel(BatchDev b, const int64_t *R, const uint8_t *statu
     }
 }
 
-// ---- minibatch gather: rows idx[r] (-1 = padding) of X into Xb and, transposed,
-// XbT ([1024][rows]), and of L into Lb; counts the valid labels into *count.
-// One block per 64 x 64 tile (grid: 16 column tiles x rows / 64 row tiles):
-// 16-byte loads and row-major stores, the transposed stores as 16-byte runs
-// of 8 rows, read column-wise from a shared-memory copy of the tile.
-constexpr int kTT = 64;
-constexpr int kTP = kTT + 8; // row pitch of a shared tile (u16): 16-byte aligned rows
-
-__device__ __forceinline__ void store_tile_t(const unsigned short (*t)[kTP], __nv_bfloat16 *out, int64_t ld,
-                                             int64_t c0, int64_t r0)
-{
-    // out[(c0 + c) * ld + r0 + 8 rc + i] = t[8 rc + i][c]: a warp writes 32 columns
-    for (int e = threadIdx.x; e < kTT * kTT / 8; e += blockDim.x) {
-        const int c = e % kTT, rc = e / kTT;
-        uint4 v;
-        unsigned short *h = reinterpret_cast<unsigned short *>(&v);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) h[i] = t[8 * rc + i][c];
-        *reinterpret_cast<uint4 *>(out + (c0 + c) * ld + r0 + 8 * rc) = v;
-    }
-}
-
+// ---- minibatch gather: rows idx[r] (-1 = padding) of X into Xb and of L into Lb;
+// counts the valid labels into *count.  A warp per row: 2 KB of X and 256 bytes of
+// labels in 16-byte pieces, four loads in flight per lane.  Bound by memory (34 MB
+// for 8,192 rows); with a transposed copy for the weight gradients it took 13 us,
+// 7.1 us now.
 __global__ void __launch_bounds__(256) gather_kernel(const __nv_bfloat16 *X, const float *L, const int64_t *idx,
-                                                     int rows, __nv_bfloat16 *Xb, __nv_bfloat16 *XbT, float *Lb,
-                                                     float *count)
+                                                     int rows, __nv_bfloat16 *Xb, float *Lb, float *count)
 {
-    __shared__ __align__(16) unsigned short t[kTT][kTP];
-    static_assert(kTT * kTT / 8 == 2 * 256, "two 16-byte loads per thread");
-    const int c0 = blockIdx.x * kTT, r0 = blockIdx.y * kTT;
-    uint4 v[2];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int e = threadIdx.x + 256 * j, r = e / (kTT / 8), part = e % (kTT / 8);
-        const int64_t src = idx[r0 + r];
-        v[j] = src >= 0 ? *reinterpret_cast<const uint4 *>(X + src * XW + c0 + 8 * part) : make_uint4(0, 0, 0, 0);
-    }
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int e = threadIdx.x + 256 * j, r = e / (kTT / 8), part = e % (kTT / 8);
-        *reinterpret_cast<uint4 *>(Xb + (int64_t)(r0 + r) * XW + c0 + 8 * part) = v[j];
-        *reinterpret_cast<uint4 *>(&t[r][8 * part]) = v[j];
-    }
-    if (XbT) {
-        __syncthreads();
-        store_tile_t(t, XbT, rows, c0, r0);
-    }
-    if (blockIdx.x != 0) return;
-    // the tile's labels: 64 rows x 16 float4
-    static_assert(kTT * NCH / 4 == 4 * 256, "four label loads per thread");
-    float4 y[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int e = threadIdx.x + 256 * j, r = e / (NCH / 4), q = e % (NCH / 4);
-        const int64_t src = idx[r0 + r];
-        y[j] = src >= 0 ? *reinterpret_cast<const float4 *>(L + src * NCH + 4 * q) : make_float4(-1.f, -1.f, -1.f, -1.f);
-    }
+    const int lane = threadIdx.x & 31;
+    const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
+    __shared__ float part[8];
     float cnt = 0.0f;
+    if (r < rows) {
+        const int64_t src = idx[r];
+        const uint4 *x = reinterpret_cast<const uint4 *>(X + src * XW);
+        uint4 *o = reinterpret_cast<uint4 *>(Xb + (int64_t)r * XW);
+        constexpr int N = XW / 8 / 32;
+        uint4 v[N];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int e = threadIdx.x + 256 * j, r = e / (NCH / 4), q = e % (NCH / 4);
-        *reinterpret_cast<float4 *>(Lb + (int64_t)(r0 + r) * NCH + 4 * q) = y[j];
-        cnt += (y[j].x >= 0.0f) + (y[j].y >= 0.0f) + (y[j].z >= 0.0f) + (y[j].w >= 0.0f);
+        for (int i = 0; i < N; ++i) v[i] = src >= 0 ? x[lane + 32 * i] : make_uint4(0, 0, 0, 0);
+        const float2 y = src >= 0 ? reinterpret_cast<const float2 *>(L + src * NCH)[lane] : make_float2(-1.f, -1.f);
+#pragma unroll
+        for (int i = 0; i < N; ++i) o[lane + 32 * i] = v[i];
+        reinterpret_cast<float2 *>(Lb + (int64_t)r * NCH)[lane] = y;
+        cnt = (float)((y.x >= 0.0f) + (y.y >= 0.0f));
     }
     for (int off = 16; off > 0; off >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, off);
-    if ((threadIdx.x & 31) == 0 && cnt > 0.0f) atomicAdd(count, cnt);
-}
-
-// ---- masked mean-squared error and its gradient dY ([rows][64]) and dY^T
-// ([64][rows]); one block per 64 rows
-__global__ void __launch_bounds__(256) loss_kernel(const float *Y, const float *Lb, int rows, const float *count,
-                                                   __nv_bfloat16 *dY, __nv_bfloat16 *dYT, float *loss_sum)
-{
-    __shared__ __align__(16) unsigned short t[kTT][kTP];
-    __shared__ float part[8];
-    static_assert(kTT * NCH / 4 == 4 * 256, "four float4 per thread");
-    const int r0 = blockIdx.x * kTT;
-    float4 yv[4], lv[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int64_t i = (int64_t)r0 * NCH + 4 * (threadIdx.x + 256 * j);
-        yv[j] = *reinterpret_cast<const float4 *>(Y + i);
-        lv[j] = *reinterpret_cast<const float4 *>(Lb + i);
-    }
-    const float inv = 1.0f / fmaxf(*count, 1.0f);
-    float acc = 0.0f;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int e = threadIdx.x + 256 * j, r = e / (NCH / 4), c = 4 * (e % (NCH / 4));
-        const float yy[4] = {yv[j].x, yv[j].y, yv[j].z, yv[j].w}, ll[4] = {lv[j].x, lv[j].y, lv[j].z, lv[j].w};
-        unsigned short g[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float d = ll[q] >= 0.0f ? yy[q] - ll[q] : 0.0f;
-            acc += d * d;
-            g[q] = __bfloat16_as_ushort(__float2bfloat16_rn(2.0f * d * inv));
-            t[r][c + q] = g[q];
-        }
-        uint2 w;
-        w.x = (unsigned)g[0] | ((unsigned)g[1] << 16);
-        w.y = (unsigned)g[2] | ((unsigned)g[3] << 16);
-        *reinterpret_cast<uint2 *>(dY + (int64_t)(r0 + r) * NCH + c) = w;
-    }
-    __syncthreads();
-    store_tile_t(t, dYT, rows, 0, r0);
-    // one atomic per block: warp sums, then the block's warps
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+    if (lane == 0) part[threadIdx.x >> 5] = cnt;
     __syncthreads();
     if (threadIdx.x == 0) {
-        float tot = 0.0f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += part[w];
-        atomicAdd(loss_sum, tot * inv);
+        float t = 0.0f;
+        for (int w = 0; w < 8; ++w) t += part[w];
+        if (t > 0.0f) atomicAdd(count, t); // whole numbers: the order does not matter
     }
 }
 
 // ---- the gradients of one minibatch, and AdamW (decoupled weight decay on
 // weights only) with a refresh of the bf16 copies.
 // A weight gradient is the sum, in slice order, of the split-K slices its
-// GEMM stored (deterministic, no atomics); a bias gradient is the row sum of
-// the layer's transposed output gradient dT ([out][rows] bf16), taken by one
-// block per bias (16-byte loads, a fixed shuffle tree per warp, the warps'
-// sums in warp order).  Blocks [0, bias_blocks) take the biases, the others
-// four weights per thread.
+// GEMM stored (deterministic, no atomics); a bias gradient is the sum, in a fixed
+// order, of the partial sums that the chain kernel left (32 rows each), and so is
+// the loss.  Blocks [0, bias_blocks) take 32 of those columns each, the others four
+// weights per thread.
 struct GradSegs {
     float *W[4], *m[4], *v[4], *g[4];  // weights [out][in] (and moments, gradient out)
     float *b[4], *mb[4], *vb[4], *gb[4];
     __nv_bfloat16 *Wb[4], *WbT[4];
     const float *part[4];              // [z][out * in] slices
-    const __nv_bfloat16 *dT[4];        // [out][rows]
+    const float *bias_part;            // [rows / 32][kPartCols]
+    float *loss;                       // the minibatch's loss is added
     int64_t woff[5];                   // weight index ranges in the concatenation (multiples of 4)
     int boff[5];                       // bias index ranges
     int z[4], rows_w[4], cols_w[4];
-    int rows;                          // minibatch rows (a multiple of 8)
+    int rows;                          // minibatch rows (a multiple of 32)
     int bias_blocks;
 };
 
@@ -228,30 +149,25 @@ __global__ void __launch_bounds__(256) grad_adamw_kernel(GradSegs a, float lr, f
                                                          float c1, float c2, float wd)
 {
     if ((int)blockIdx.x < a.bias_blocks) {
-        __shared__ float part[8];
-        const int j = blockIdx.x, lane = threadIdx.x & 31;
-        int k = 0;
-        while (k < 3 && j >= a.boff[k + 1]) ++k;
-        const int o = j - a.boff[k];
-        const uint4 *row = reinterpret_cast<const uint4 *>(a.dT[k] + (int64_t)o * a.rows);
+        __shared__ float part[8][32];
+        const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, j = blockIdx.x * 32 + lane;
         float acc = 0.0f;
 #pragma unroll 4
-        for (int q = threadIdx.x; q < a.rows / 8; q += blockDim.x) {
-            const uint4 v = row[q];
-            const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float2 f = __bfloat1622float2(h[i]);
-                acc += f.x + f.y;
-            }
-        }
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) part[threadIdx.x >> 5] = acc;
+        for (int t = wp; t < a.rows / 32 && j < kBiasCols + 2; t += 8)
+            acc += a.bias_part[(int64_t)t * kPartCols + j];
+        part[wp][lane] = acc;
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (wp == 0) {
+            int k = 0;
+            while (k < 3 && j >= a.boff[k + 1]) ++k;
+            const int o = j - a.boff[k];
             float g = 0.0f;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) g += part[w];
-            if (UPDATE)
+#pragma unroll
+            for (int w = 0; w < 8; ++w) g += part[w][lane];
+            if (j >= kBiasCols) { // the last block: two columns of losses
+                g += __shfl_down_sync(0xffffffffu, g, 1);
+                if (lane == 0) *a.loss += g;
+            } else if (UPDATE)
                 adam_step(a.b[k][o], a.mb[k][o], a.vb[k][o], g, lr, b1, b2, eps, c1, c2, 0.0f);
             else
                 a.gb[k][o] = g;
@@ -535,14 +451,14 @@ constexpr int64_t kInferRows = (int64_t)1 << 22;
 struct Work {
     int rows;
     void *block;
-    __nv_bfloat16 *Xb, *XbT, *Z[3], *H[3], *HT[3], *dY, *dYT, *dZ[3], *dZT[3];
-    float *Lb, *Y, *count, *loss;
+    __nv_bfloat16 *Xb, *Z, *H[3], *dY, *dZ[3];
+    float *Lb, *Y, *count, *loss, *bias_part;
     float *part[4]; // per layer, the split-K slices of its weight gradient (training)
     int z[4];       // slices per layer
     int32_t *err;
 };
 
-// Weight-gradient GEMMs dW = dT x in^T contract over the minibatch rows: K is
+// Weight-gradient GEMMs dW = d^T in contract over the minibatch rows: K is
 // split so that the tiles times the splits cover the SMs about once, with at
 // least two 64-row steps per split; each split stores its own slice and the
 // slices are summed in order (deterministic, no atomics).
@@ -580,8 +496,9 @@ int work_alloc(Work &w, int rows, bool train, cudaStream_t s, int xw = XW, int n
     if (n_sm < 1) n_sm = 1;
     size_t part = 0;
     for (int l = 0; train && l < NL; ++l) part += 4 * dw_part_floats(l, rows, n_sm);
-    size_t bytes = 2 * r * xw * (train ? 2 : 1) + 3 * 2 * r * 256 * (train ? 6 : 1) + 4 * r * 64 * (train ? 2 : 1) +
-                   2 * 2 * r * 64 + 64 * 256 + part + 256;
+    const size_t bias_part = train ? 4 * (r / 32) * kPartCols : 0;
+    size_t bytes = 2 * r * xw + 2 * r * 256 * (train ? 7 : 3) + 4 * r * 64 + (train ? 2 * r * 64 : 0) + bias_part +
+                   64 * 256 + part + 256;
     if (cudaMallocAsync(&w.block, bytes, s) != cudaSuccess) {
         cudaGetLastError();
         return PAAM_E_NOMEM;
@@ -593,21 +510,17 @@ int work_alloc(Work &w, int rows, bool train, cudaStream_t s, int xw = XW, int n
         return q;
     };
     w.Xb = (__nv_bfloat16 *)take(2 * r * xw);
-    if (train) w.XbT = (__nv_bfloat16 *)take(2 * r * xw);
     for (int l = 0; l < 3; ++l) {
+        if (train) w.dZ[l] = (__nv_bfloat16 *)take(2 * r * 256);
         w.H[l] = (__nv_bfloat16 *)take(2 * r * 256);
-        if (train) {
-            w.Z[l] = (__nv_bfloat16 *)take(2 * r * 256);
-            w.HT[l] = (__nv_bfloat16 *)take(2 * r * 256);
-            w.dZ[l] = (__nv_bfloat16 *)take(2 * r * 256);
-            w.dZT[l] = (__nv_bfloat16 *)take(2 * r * 256);
-        }
     }
-    w.Y = (float *)take(4 * r * 64);
     if (train) {
+        w.Z = (__nv_bfloat16 *)take(2 * r * 256);
         w.Lb = (float *)take(4 * r * 64);
         w.dY = (__nv_bfloat16 *)take(2 * r * 64);
-        w.dYT = (__nv_bfloat16 *)take(2 * r * 64);
+        w.bias_part = (float *)take(bias_part);
+    } else {
+        w.Y = (float *)take(4 * r * 64);
     }
     for (int l = 0; train && l < NL; ++l) {
         w.part[l] = (float *)take(4 * dw_part_floats(l, rows, n_sm));
@@ -617,16 +530,6 @@ int work_alloc(Work &w, int rows, bool train, cudaStream_t s, int xw = XW, int n
     w.loss = (float *)take(4);
     w.err = (int32_t *)take(4);
     return PAAM_OK;
-}
-
-// Column tile for a minibatch GEMM: the widest that still gives every SM a
-// tile (minibatches of a few thousand rows have few row tiles).
-int bn_for(int M, int N, int n_sm)
-{
-    const int mt = (M + 127) / 128;
-    for (int bn = 256; bn >= 64; bn /= 2)
-        if (N % bn == 0 && mt * (N / bn) >= n_sm) return bn;
-    return 64;
 }
 
 TcGemm gemm(const __nv_bfloat16 *A, int lda, int a_rows, const __nv_bfloat16 *B, int ldb, int b_rows, int K)
@@ -651,8 +554,7 @@ int input_width(const paam_batch *b)
     return w < XW ? w : XW;
 }
 
-// X (rows of w.Xb, kx columns) through the network into w.Y; keeps Z, H, H^T
-// when training.  kx < 1024 reads only the first kx input columns of layer 1:
+// X (rows of w.Xb, kx columns) through the network into w.Y.  kx < 1024 reads only the first kx input columns of layer 1:
 // exact when the remaining feature columns are zero (chain slots past every
 // system's chains), since their products add nothing to the fp32 sums.
 // With score != NULL the output layer writes, per row, the largest
@@ -667,7 +569,7 @@ struct ScoreOut {
     const int32_t *sys_list; // rows' systems through this list (NULL: consecutive from sys0)
 };
 
-int forward(const paam_model *m, Work &w, const __nv_bfloat16 *X, int kx, bool train, cudaStream_t s,
+int forward(const paam_model *m, Work &w, const __nv_bfloat16 *X, int kx, cudaStream_t s,
             const ScoreOut *so = nullptr)
 {
     const int rows = w.rows;
@@ -678,13 +580,8 @@ int forward(const paam_model *m, Work &w, const __nv_bfloat16 *X, int kx, bool t
         g.ep.M = rows;
         g.ep.N = OUT[l];
         g.ep.bias = m->bias[l];
-        g.ep.Z = train ? w.Z[l] : nullptr;
-        g.ep.ldz = OUT[l];
         g.ep.H = w.H[l];
         g.ep.ldh = OUT[l];
-        g.ep.HT = train ? w.HT[l] : nullptr;
-        g.ep.ldht = rows;
-        if (train) g.bn = bn_for(rows, OUT[l], m->ctx->n_sm);
         int rc = tc_gemm(g, w.err, s);
         if (rc != PAAM_OK) return rc;
     }
@@ -695,7 +592,6 @@ int forward(const paam_model *m, Work &w, const __nv_bfloat16 *X, int kx, bool t
     g.ep.bias = m->bias[3];
     g.ep.C = w.Y;
     g.ep.ldc = OUT[3];
-    if (train) g.bn = bn_for(rows, OUT[3], m->ctx->n_sm);
     if (so) {
         PAAM_CUDA_TRY(cudaMemsetAsync(so->score, 0, 4 * (size_t)rows, s));
         g.ep.mode = TC_EPI_ROWMAX;
@@ -739,27 +635,34 @@ struct Branches {
     }
 };
 
-// The masked MSE's gradients as the backward GEMMs leave them: per layer, the
-// split-K slices of the weight gradient in w.part[l] and the transposed output
-// gradient (dY^T, dZ^T) whose row sums are the bias gradient; grad_adamw
+// A minibatch's chain (forward, loss, input gradients) and, on what it leaves, every
+// layer's weight gradient dW = d^T in as split-K slices in w.part[l].  grad_adamw
 // finishes them.
-int backward(paam_model *m, Work &w, cudaStream_t s)
+// In a captured step the weight gradients are branches beside each other.
+int gradients(paam_model *m, Work &w, cudaStream_t s)
 {
     const int rows = w.rows, sm = m->ctx->n_sm;
-    loss_kernel<<<rows / kTT, 256, 0, s>>>(w.Y, w.Lb, rows, w.count, w.dY, w.dYT, w.loss);
-    PAAM_CUDA_TRY(cudaGetLastError());
-    paam_count_launch();
-    // output layer: dW4 = dY^T H3, db4 = column sums of dY, dH3 = dY W4 (then the GELU derivative)
-    const __nv_bfloat16 *dT = w.dYT; // [OUT[l]][rows]
-    const __nv_bfloat16 *d = w.dY;   // [rows][OUT[l]]
-    // in a captured step each weight gradient is a branch beside the input gradients,
-    // which are what the next layer waits for: the step's chain is 11 kernels, not 14
+    TrainChain c = {};
+    c.rows = rows;
+    for (int l = 0; l < NL; ++l) c.bias[l] = m->bias[l];
+    for (int l = 0; l < 3; ++l) c.H[l] = w.H[l], c.dZ[l] = w.dZ[l];
+    c.Z = w.Z;
+    c.dY = w.dY;
+    c.bias_part = w.bias_part;
+    c.L = w.Lb;
+    c.count = w.count;
+    c.err = w.err;
+    const __nv_bfloat16 *W[NL] = {m->Wb[0], m->Wb[1], m->Wb[2], m->Wb[3]};
+    const __nv_bfloat16 *WT[NL] = {m->WbT[0], m->WbT[1], m->WbT[2], m->WbT[3]};
+    int rc = paam_train_chain(c, w.Xb, W, WT, s);
+    if (rc != PAAM_OK) return rc;
     Branches br(s);
     std::vector<cudaGraphNode_t> here, end, ends;
-    for (int l = 3; l >= 0; --l) {
-        if (br.now(here) != PAAM_OK) return PAAM_E_CUDA;
-        const __nv_bfloat16 *inT = l == 0 ? w.XbT : w.HT[l - 1];
-        TcGemm g = gemm(dT, rows, OUT[l], inT, rows, IN[l], rows);
+    if (br.now(here) != PAAM_OK) return PAAM_E_CUDA;
+    for (int l = 0; l < NL; ++l) { // the largest first
+        if (l > 0 && br.follow(here) != PAAM_OK) return PAAM_E_CUDA;
+        TcGemm g = gemm(l == 3 ? w.dY : w.dZ[l], OUT[l], OUT[l], l == 0 ? w.Xb : w.H[l - 1], IN[l], IN[l], rows);
+        g.mn = 1; // both operands have the rows outermost
         const DwPlan dp = dw_plan(OUT[l], IN[l], rows, sm);
         g.ep.mode = TC_EPI_STORE_F32;
         g.ep.M = OUT[l];
@@ -769,27 +672,10 @@ int backward(paam_model *m, Work &w, cudaStream_t s)
         g.ep.split_stride = (int64_t)OUT[l] * IN[l];
         g.splits = dp.splits;
         g.bn = dp.bn;
-        int rc = tc_gemm(g, w.err, s);
+        rc = tc_gemm(g, w.err, s);
         if (rc != PAAM_OK) return rc;
         if (br.now(end) != PAAM_OK) return PAAM_E_CUDA;
         ends.insert(ends.end(), end.begin(), end.end());
-        if (l == 0) break;
-        if (br.follow(here) != PAAM_OK) return PAAM_E_CUDA;
-        TcGemm h = gemm(d, OUT[l], rows, m->WbT[l], OUT[l], IN[l], OUT[l]);
-        h.ep.mode = TC_EPI_DGELU;
-        h.ep.M = rows;
-        h.ep.N = IN[l];
-        h.ep.Zin = w.Z[l - 1];
-        h.ep.ldzin = IN[l];
-        h.ep.H = w.dZ[l - 1];
-        h.ep.ldh = IN[l];
-        h.ep.HT = w.dZT[l - 1];
-        h.ep.ldht = rows;
-        h.bn = bn_for(rows, IN[l], sm);
-        rc = tc_gemm(h, w.err, s);
-        if (rc != PAAM_OK) return rc;
-        dT = w.dZT[l - 1];
-        d = w.dZ[l - 1];
     }
     return br.follow(ends);
 }
@@ -807,7 +693,6 @@ int grad_adamw(paam_model *m, const Work &w, const paam_train_opts *o, float c1,
         a.Wb[l] = m->Wb[l], a.WbT[l] = m->WbT[l];
         a.part[l] = w.part[l];
         a.z[l] = w.z[l];
-        a.dT[l] = l == 3 ? w.dYT : w.dZT[l];
         a.rows_w[l] = OUT[l], a.cols_w[l] = IN[l];
         a.woff[l] = off;
         a.boff[l] = boff;
@@ -817,7 +702,10 @@ int grad_adamw(paam_model *m, const Work &w, const paam_train_opts *o, float c1,
     a.woff[NL] = off;
     a.boff[NL] = boff;
     a.rows = w.rows;
-    a.bias_blocks = boff; // one block per bias
+    a.bias_part = w.bias_part;
+    static_assert(kBiasCols % 32 == 0 && kPartCols == kBiasCols + 32, "32 biases per block, the losses in one more");
+    a.loss = w.loss;
+    a.bias_blocks = kPartCols / 32;
     const unsigned grid = (unsigned)a.bias_blocks + grid_for(off / 4, 256, m->ctx->n_sm);
     if (o)
         grad_adamw_kernel<true><<<grid, 256, 0, s>>>(a, o->lr, o->beta1, o->beta2, o->adam_eps, c1, c2,
@@ -891,11 +779,10 @@ int enqueue_step(paam_model *m, Work &w, const __nv_bfloat16 *X, const float *L,
 {
     const int rows = w.rows;
     PAAM_CUDA_TRY(cudaMemsetAsync(w.count, 0, 4, s));
-    gather_kernel<<<dim3(XW / kTT, rows / kTT), 256, 0, s>>>(X, L, idx, rows, w.Xb, w.XbT, w.Lb, w.count);
+    gather_kernel<<<(rows + 7) / 8, 256, 0, s>>>(X, L, idx, rows, w.Xb, w.Lb, w.count);
     PAAM_CUDA_TRY(cudaGetLastError());
     paam_count_launch();
-    int rc = forward(m, w, w.Xb, XW, true, s);
-    if (rc == PAAM_OK) rc = backward(m, w, s);
+    int rc = gradients(m, w, s);
     if (rc == PAAM_OK) rc = grad_adamw(m, w, o, c1, c2, s);
     return rc;
 }
@@ -916,7 +803,7 @@ struct StepGraph {
     }
 };
 
-constexpr int kGatherArgs = 8, kAdamArgs = 8; // argument counts of gather_kernel, grad_adamw_kernel
+constexpr int kGatherArgs = 7, kAdamArgs = 8; // argument counts of gather_kernel, grad_adamw_kernel
 
 int capture_step(StepGraph &g, paam_model *m, Work &w, const __nv_bfloat16 *X, const float *L, const int64_t *idx,
                  const paam_train_opts *o, float c1, float c2, cudaStream_t s)
@@ -1109,7 +996,7 @@ int infer_rank(paam_ctx *ctx, const paam_model *m, const paam_batch *b, const in
         wc.rows = (int)items;
         rc = paam_launch_features(b, ranks, K, nmax, s0, items, n_buckets, kappa_ns, kx, wc.Xb, s, sys_list);
         const ScoreOut so = {sc + s0 * K, b->sys_chain_off, s0, K, sys_list};
-        if (rc == PAAM_OK) rc = forward(m, wc, wc.Xb, kx, false, s, &so);
+        if (rc == PAAM_OK) rc = forward(m, wc, wc.Xb, kx, s, &so);
     }
     if (rc == PAAM_OK) {
         topk_kernel<<<(unsigned)((n_list + 7) / 8), 256, 0, s>>>(sc, n_list, K, n_pinned, top_k, ranked, sys_list,
@@ -1283,7 +1170,7 @@ extern "C" int paam_surrogate_predict(paam_ctx *ctx, const paam_model *m, const 
         wc.rows = (int)((s0 + chunk <= b->n_sys) ? chunk : b->n_sys - s0);
         wc.Y = pred + s0 * NCH;
         rc = paam_launch_features(b, nullptr, 1, 0, s0, wc.rows, n_buckets, kappa_ns, kx, wc.Xb, s);
-        if (rc == PAAM_OK) rc = forward(m, wc, wc.Xb, kx, false, s);
+        if (rc == PAAM_OK) rc = forward(m, wc, wc.Xb, kx, s);
     }
     int32_t herr = 0;
     if (cudaMemcpyAsync(&herr, w.err, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess) rc = PAAM_E_CUDA;
@@ -1317,13 +1204,11 @@ extern "C" int paam_surrogate_grad(paam_ctx *ctx, paam_model *m, const void *X, 
         cudaMemsetAsync(w.loss, 0, 4, s) != cudaSuccess)
         rc = PAAM_E_CUDA;
     if (rc == PAAM_OK) {
-        gather_kernel<<<dim3(XW / kTT, rows / kTT), 256, 0, s>>>((const __nv_bfloat16 *)X, L, idx, rows, w.Xb,
-                                                                 w.XbT, w.Lb, w.count);
+        gather_kernel<<<(rows + 7) / 8, 256, 0, s>>>((const __nv_bfloat16 *)X, L, idx, rows, w.Xb, w.Lb, w.count);
         if (cudaGetLastError() != cudaSuccess) rc = PAAM_E_CUDA;
         paam_count_launch();
     }
-    if (rc == PAAM_OK) rc = forward(m, w, w.Xb, XW, true, s);
-    if (rc == PAAM_OK) rc = backward(m, w, s);
+    if (rc == PAAM_OK) rc = gradients(m, w, s);
     if (rc == PAAM_OK) rc = grad_adamw(m, w, nullptr, 1.0f, 1.0f, s);
     size_t o = 0;
     for (int l = 0; l < NL && rc == PAAM_OK; ++l) {

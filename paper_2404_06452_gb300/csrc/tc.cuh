@@ -65,6 +65,69 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64
     return true;
 }
 
+// ---- a pair of CTAs (cluster) --------------------------------------------------
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+// every thread of the cluster's CTAs: what each did before is seen by all after
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// the shared-memory address in CTA `rank` of what `saddr` is in this one
+__device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+    return r;
+}
+
+__device__ __forceinline__ void st_cluster(uint32_t addr, uint4 v)
+{
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
+}
+
+// arrive at a barrier of any CTA of the cluster (address from map_rank)
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+
+// mbar_wait for arrivals from other CTAs of the cluster
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t *bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok)
+                 : "r"(smem_u32(bar)), "r"(parity)
+                 : "memory");
+    return ok != 0;
+}
+
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity, uint64_t limit_ns)
+{
+    if (mbar_try_wait_cluster(bar, parity)) return true;
+    const uint64_t t0 = global_ns();
+    while (!mbar_try_wait_cluster(bar, parity))
+        if (global_ns() - t0 > limit_ns) return false;
+    return true;
+}
+
+// generic-proxy writes to shared memory, of this CTA or another of the cluster,
+// become visible to the async proxy
+__device__ __forceinline__ void fence_proxy_async_cluster()
+{
+    asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
+}
+
 // ---- TMA ---------------------------------------------------------------------
 // 2-D tile load into shared memory; completion is signalled on `bar` as
 // transaction bytes.  x is the inner (contiguous) coordinate.
@@ -145,6 +208,15 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar)
                  : "memory");
 }
 
+// The same at the barrier in the same place of every CTA in `mask` of the cluster.
+__device__ __forceinline__ void mma_commit_multicast(uint64_t *bar, uint16_t mask)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+                     smem_u32(bar)),
+                 "h"(mask)
+                 : "memory");
+}
+
 // Instruction descriptor of kind::f16: fp32 accumulator, bf16 A and B, both
 // K-major, M x N tile.
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N)
@@ -162,6 +234,24 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr)
     d |= (uint64_t)(1024 >> 4) << 32; // stride byte offset between 8-row groups
     d |= (uint64_t)1 << 46;          // descriptor version
     d |= (uint64_t)2 << 61;          // 128-byte swizzle
+    return d;
+}
+
+// The same with A and B "MN-major": stored with the contraction index outermost
+// (bits 15 and 16: transposed operands).
+__host__ __device__ constexpr uint32_t idesc_bf16_mn(int M, int N) { return idesc_bf16(M, N) | (1u << 15) | (1u << 16); }
+
+// Shared-memory matrix descriptor for an MN-major tile stored with the 128-byte
+// swizzle as boxes of 64 contraction rows x 64 bf16 (8 KB each, one after another
+// along M or N): 8-row groups of the contraction 1024 bytes apart, boxes 8192.
+__device__ __forceinline__ uint64_t desc_mn_sw128(uint32_t saddr)
+{
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(8192 >> 4) << 16; // leading byte offset: the next 64 of M or N
+    d |= (uint64_t)(1024 >> 4) << 32; // stride byte offset: the next 8 contraction rows
+    d |= (uint64_t)1 << 46;           // descriptor version
+    d |= (uint64_t)2 << 61;           // 128-byte swizzle
     return d;
 }
 
