@@ -1,8 +1,9 @@
 // gelu.cuh -- the surrogate network's activation on the GPU, used by the
-// GEMM epilogues (mlp_gemm.cu).
+// epilogues of mlp_gemm.cu, mlp_train.cu and mlp_infer.cu.
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stdint.h>
 
 namespace paam_gelu {
 
@@ -38,6 +39,51 @@ __device__ __forceinline__ float gelu_gate(float z)
 }
 
 __device__ __forceinline__ float gelu(float z) { return z * gelu_gate(z); }
+
+// The same for two values, with the paired fp32 instructions (each half rounds as the
+// single one does: the results' bits are the same)
+__device__ __forceinline__ uint64_t pack2(float x, float y)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+
+__device__ __forceinline__ float2 unpack2(uint64_t v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+__device__ __forceinline__ float2 gelu2(uint64_t z)
+{
+    constexpr float k0 = -2.3022082f, k1 = -0.10294324f;
+    const float2 w = unpack2(mul2(z, fma2(pack2(k1, k1), mul2(z, z), pack2(k0, k0))));
+    const float2 d = unpack2(add2(pack2(1.0f, 1.0f), pack2(ex2_approx(fminf(w.x, 126.0f)), ex2_approx(fminf(w.y, 126.0f)))));
+    return unpack2(mul2(z, pack2(rcp_approx(d.x), rcp_approx(d.y))));
+}
 
 // d/dz z s(z), s = sigmoid(2u): s + z s (1 - s) d(2u)/dz, d(2u)/dz = c0 + 3 c1 z^2
 __device__ __forceinline__ float gelu_grad(float z)

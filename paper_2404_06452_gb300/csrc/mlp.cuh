@@ -65,16 +65,13 @@ bool tc_make_map(CUtensorMap *m, const __nv_bfloat16 *base, int rows, int cols, 
 // [rows][1024], the layers' bf16 weights W [out][in] and WT [in][out] and the fp32
 // labels L [rows][64] (< 0: none; *count of them valid); writes the activations H and
 // the gradients dZ [rows][256] and dY [rows][64] (and Z, its own), and
-// leaves each bias gradient as rows / 32 sums of 32 rows in bias_part ([rows / 32]
-// [kPartCols], the layers' biases one after another) and behind them the loss's, two
-// columns (one per half of the outputs).
-constexpr int kBiasCols = 3 * 256 + 64, kPartCols = kBiasCols + 32;
+// leaves the loss as rows / 16 sums in loss_part.
 struct TrainChain {
     int rows;
     const float *bias[4];
     __nv_bfloat16 *Z, *H[3], *dY, *dZ[3];
     const float *L, *count;
-    float *bias_part;
+    float *loss_part;
     int32_t *err;
 };
 int paam_train_chain(const TrainChain &c, const __nv_bfloat16 *X, const __nv_bfloat16 *const (&W)[4],

@@ -13,7 +13,7 @@
 // gradient GEMMs contract over, by TMA from the operand tiles (those GEMMs read them
 // transposed, so nothing is stored transposed), and the first layer's pre-activations,
 // which come back for its gradient (the other two layers' stay in shared memory).
-// Bias gradients leave as sums of 32 rows, taken by a halving exchange in each warp.
+// The loss leaves as sums of 32 rows and half of the columns.
 //
 //   phase 0 1 2   H_l = gelu(H_(l-1) W_l^T + b_l)
 //         3       Y = H_2 W_3^T + b_3, loss, dY
@@ -26,7 +26,7 @@
 // epilogues are before either's next MMAs.  The sums are those of a kernel per layer,
 // in the same order.  Bound by the epilogues: the activation's two special-function
 // results per element take 1 us per phase.  8,192 rows: seven kernels 75 us, one CTA
-// per 128 rows 51-60, a pair 45 us (about 11,000 cycles per phase, 1,200 of them MMAs,
+// per 128 rows 51-60, a pair 44 us (about 11,000 cycles per phase, 1,200 of them MMAs,
 // 2,900 arithmetic, 4,000 the operand writes into both CTAs and the fence behind them).
 #include "gelu.cuh"
 #include "mlp.cuh"
@@ -58,45 +58,11 @@ struct ChainMaps {
     CUtensorMap Z;          // the first layer's pre-activations
 };
 
-// A thread's 32 columns col0.. of tile row `row` in a tile of 64-column blocks
-__device__ __forceinline__ uint32_t piece_at(uint32_t tile, int row, int col0, int k)
-{
-    return tile + (uint32_t)((col0 >> 6) * kA + row * 128 + (((((col0 & 63) >> 3) + k) ^ (row & 7)) << 4));
-}
-
-__device__ __forceinline__ void put_piece(uint32_t at, uint4 v)
-{
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
-
 __device__ __forceinline__ uint4 get_piece(uint32_t at)
 {
     uint4 v;
     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
     return v;
-}
-
-// The sums over the warp's 32 rows of its 32 columns, column `lane` in each lane: in
-// each step a lane keeps half of its columns and hands the other half over.
-__device__ __forceinline__ float column_sum(const __nv_bfloat162 (&out)[16], int lane)
-{
-    float v[32];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const float2 f = __bfloat1622float2(out[i]);
-        v[2 * i] = f.x;
-        v[2 * i + 1] = f.y;
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const bool up = (lane & off) != 0;
-#pragma unroll
-        for (int i = 0; i < off; ++i) {
-            const float give = up ? v[i] : v[i + off], keep = up ? v[i + off] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, off);
-        }
-    }
-    return v[0];
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
@@ -189,6 +155,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     ok = false;
                     break;
                 }
+                tc::fence_after_sync();
                 if (p == 5) { // Z_2's tile has been read: Z_0 comes back into it
                     tc::bulk_wait_all();
                     tc::mbar_expect_tx(zbar, kZ);
@@ -204,13 +171,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     ok = false;
                     break;
                 }
-                tc::fence_after_sync();
                 const uint32_t st = tc::smem_u32(smem + s * kStage);
-                const uint32_t a = p == 0 ? st : tc::smem_u32(hs + kb * kA), w = st + kA;
+                const uint64_t a = tc::desc_sw128(p == 0 ? st : tc::smem_u32(hs + kb * kA));
+                const uint64_t w = tc::desc_sw128(st + kA);
 #pragma unroll
                 for (int j = 0; j < BK / 16; ++j)
-                    tc::mma_bf16(tmem, tc::desc_sw128(a + 32 * j), tc::desc_sw128(w + 32 * j), idesc,
-                                 (kb > 0 || j > 0) ? 1u : 0u);
+                    tc::mma_bf16(tmem, a + 2 * j, w + 2 * j, idesc, (kb > 0 || j > 0) ? 1u : 0u);
                 tc::mma_commit(&empty[s]);
             }
             if (!ok) break;
@@ -268,15 +234,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const float4 b = __ldg(b4 + i);
-                        const float a0 = __uint_as_float(v[4 * i]) + b.x, a1 = __uint_as_float(v[4 * i + 1]) + b.y;
-                        const float a2 = __uint_as_float(v[4 * i + 2]) + b.z, a3 = __uint_as_float(v[4 * i + 3]) + b.w;
-                        z2[2 * i] = __floats2bfloat162_rn(a0, a1);
-                        z2[2 * i + 1] = __floats2bfloat162_rn(a2, a3);
-                        out[2 * i] = __floats2bfloat162_rn(gelu(a0), gelu(a1));
-                        out[2 * i + 1] = __floats2bfloat162_rn(gelu(a2), gelu(a3));
+                        const uint64_t za = add2(pack2(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1])), pack2(b.x, b.y));
+                        const uint64_t zc = add2(pack2(__uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3])), pack2(b.z, b.w));
+                        const float2 a0 = unpack2(za), a2 = unpack2(zc), g0 = gelu2(za), g2 = gelu2(zc);
+                        z2[2 * i] = __floats2bfloat162_rn(a0.x, a0.y);
+                        z2[2 * i + 1] = __floats2bfloat162_rn(a2.x, a2.y);
+                        out[2 * i] = __floats2bfloat162_rn(g0.x, g0.y);
+                        out[2 * i + 1] = __floats2bfloat162_rn(g2.x, g2.y);
                     }
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) put_piece(piece_at(zt, tr, here, k), zb[k]);
+                    for (int k = 0; k < 4; ++k) tc::st_shared(tc::sw128_piece(zt, tr, here, k), zb[k]);
                 } else if (p == 3) { // outputs, masked squared error and its gradient
                     const float4 *b4 = reinterpret_cast<const float4 *>(c.bias[3] + col0);
                     const float4 *l4 = reinterpret_cast<const float4 *>(c.L + row * kOut + col0);
@@ -300,12 +267,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                         out[2 * i + 1] = __floats2bfloat162_rn(g[2], g[3]);
                     }
                     for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-                    if (lane == 0) c.bias_part[(row >> 5) * kPartCols + kBiasCols + rank] = acc * inv;
+                    if (lane == 0) c.loss_part[2 * (row >> 5) + rank] = acc * inv;
                 } else { // through the activation
                     const uint32_t zt = tc::smem_u32(zs + (p == 5 ? kZ : 0));
                     uint4 zb[4];
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) zb[k] = get_piece(piece_at(zt, tr, here, k));
+                    for (int k = 0; k < 4; ++k) zb[k] = get_piece(tc::sw128_piece(zt, tr, here, k));
                     const __nv_bfloat162 *z2 = reinterpret_cast<const __nv_bfloat162 *>(zb);
                     tc::tmem_wait_ld();
 #pragma unroll
@@ -322,8 +289,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 const uint4 *o4 = reinterpret_cast<const uint4 *>(out);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const uint32_t at = piece_at(0, tr, col0, k);
-                    put_piece(hme + at, o4[k]);
+                    const uint32_t at = tc::sw128_piece(0, tr, col0, k);
+                    tc::st_shared(hme + at, o4[k]);
                     if (p < kPhases - 1) tc::st_cluster(hpeer + at, o4[k]);
                 }
             }
@@ -334,10 +301,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 tc::mbar_arrive_cluster(tc::map_rank(tc::smem_u32(ready), rank));
                 tc::mbar_arrive_cluster(ready_peer);
             }
-            // beside the next phase's MMAs: layer 6 - p's bias gradient (p = 3: the output layer's)
-            if (p > 3 || (p == 3 && cg == 0))
-                c.bias_part[(row >> 5) * kPartCols + (p == 3 ? 3 : 6 - p) * kHidden + col0 + lane] =
-                    column_sum(out, lane);
         }
     }
     __syncthreads();

@@ -65,6 +65,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64
     return true;
 }
 
+// true in one lane of the (whole) warp
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t one;
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "elect.sync _|p, 0xffffffff;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(one));
+    return one;
+}
+
 // ---- a pair of CTAs (cluster) --------------------------------------------------
 __device__ __forceinline__ uint32_t cluster_rank()
 {
@@ -146,6 +157,12 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, const void 
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
                  ::"l"(map), "r"(smem_u32(smem_src)), "r"(x), "r"(y)
                  : "memory");
+}
+
+// The tile a later tma_load_2d reads comes into L2
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *map, int x, int y)
+{
+    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
 }
 
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
@@ -255,6 +272,18 @@ __device__ __forceinline__ uint64_t desc_mn_sw128(uint32_t saddr)
     return d;
 }
 
+// The 16-byte piece k of columns col0.. (a multiple of 8) of row `row` in a K-major bf16
+// operand tile of 128 rows, blocks of 64 columns one after another, 128-byte swizzle
+__device__ __forceinline__ uint32_t sw128_piece(uint32_t tile, int row, int col0, int k)
+{
+    return tile + (uint32_t)((col0 >> 6) * 16384 + row * 128 + (((((col0 & 63) >> 3) + k) ^ (row & 7)) << 4));
+}
+
+__device__ __forceinline__ void st_shared(uint32_t at, uint4 v)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+
 // ---- TMEM -> registers ----------------------------------------------------------
 // 32 consecutive fp32 columns of this warp's 32 TMEM lanes (one row per thread).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
@@ -267,6 +296,18 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
                    "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
                    "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
                    "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                 : "r"(taddr)
+                 : "memory");
+}
+
+// 16 of them
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+                   "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+                   "=r"(r[14]), "=r"(r[15])
                  : "r"(taddr)
                  : "memory");
 }
