@@ -60,6 +60,24 @@ int tc_gemm(const TcGemm &g, int32_t *err, cudaStream_t stream);
 // of box_rows x 64 in the 128-byte swizzle, zeros outside.
 bool tc_make_map(CUtensorMap *m, const __nv_bfloat16 *base, int rows, int cols, int ld, int box_rows);
 
+// The surrogate over `rows` rows of kx features and each row's score, the largest of 0 and
+// its first n outputs, n being the chains of system sys0 + row / rows_per_sys (with
+// sys_list: of that entry of it); for kx a multiple of 64 up to 256, which has at most 16
+// chains (mlp_infer.cu).
+struct ScoreChain {
+    int rows, kx, n_sm;
+    const float *bias[4];
+    float *score;
+    const int64_t *sys_off;
+    int64_t sys0;
+    int rows_per_sys;
+    const int32_t *sys_list;
+    int32_t *err;
+};
+bool paam_score_chain_takes(int kx);
+int paam_score_chain(const ScoreChain &c, const __nv_bfloat16 *X, const __nv_bfloat16 *const (&W)[4],
+                     cudaStream_t stream);
+
 // The chain of a training step over `rows` minibatch rows (a multiple of 128):
 // forward, masked mean-squared error and input gradients (mlp_train.cu).  Reads X
 // [rows][1024], the layers' bf16 weights W [out][in] and WT [in][out] and the fp32

@@ -621,6 +621,20 @@ int forward(const paam_model *m, Work &w, const __nv_bfloat16 *X, int kx, cudaSt
             const ScoreOut *so = nullptr)
 {
     const int rows = w.rows;
+    if (so && paam_score_chain_takes(kx)) {
+        ScoreChain c = {};
+        c.rows = rows;
+        c.kx = kx;
+        c.n_sm = m->ctx->n_sm;
+        for (int l = 0; l < NL; ++l) c.bias[l] = m->bias[l];
+        c.score = so->score;
+        c.sys_off = so->sys_off;
+        c.sys0 = so->sys0;
+        c.rows_per_sys = so->K;
+        c.sys_list = so->sys_list;
+        c.err = w.err;
+        return paam_score_chain(c, X, {m->Wb[0], m->Wb[1], m->Wb[2], m->Wb[3]}, s);
+    }
     for (int l = 0; l < 3; ++l) {
         TcGemm g = l == 0 ? gemm(X, kx, rows, m->Wb[0], IN[0], OUT[0], kx)
                           : gemm(w.H[l - 1], IN[l], rows, m->Wb[l], IN[l], OUT[l], IN[l]);
@@ -1024,7 +1038,7 @@ int infer_rank(paam_ctx *ctx, const paam_model *m, const paam_batch *b, const in
     const int rows = (int)(chunk * K);
     const int kx = input_width(b);
     Work w;
-    int rc = work_alloc(w, rows, false, s, kx);
+    int rc = work_alloc(w, rows, false, s, kx, 0, !paam_score_chain_takes(kx));
     if (rc != PAAM_OK) return rc;
     float *sc = scores;
     void *tmp = nullptr;
