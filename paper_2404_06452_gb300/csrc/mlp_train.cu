@@ -19,15 +19,16 @@
 //         3       Y = H_2 W_3^T + b_3, loss, dY
 //         4 5 6   dZ_l = (dZ_(l+1) W_(l+1)) gelu'(Z_l), l = 2, 1, 0
 //
-// Warp 0 streams the operands (3 stages of 16 + 16 KB), one thread of warp 1 issues
+// Warp 0 streams the operands (3 stages of 16 + 16 KB), one lane of warp 1 issues
 // the MMAs (128 x 128 or 128 x 32 x 16, fp32 accumulator in TMEM) and the stores, 16
 // warps run the epilogues (four per TMEM lane quadrant, 32 columns each).  A phase's
 // MMAs of both CTAs are complete before either epilogue writes operand tiles, and both
 // epilogues are before either's next MMAs.  The sums are those of a kernel per layer,
 // in the same order.  Bound by the epilogues: the activation's two special-function
 // results per element take 1 us per phase.  8,192 rows: seven kernels 75 us, one CTA
-// per 128 rows 51-60, a pair 44 us (about 11,000 cycles per phase, 1,200 of them MMAs,
-// 2,900 arithmetic, 4,000 the operand writes into both CTAs and the fence behind them).
+// per 128 rows 51-60, a pair 41 us (about 10,000 cycles per phase, 1,200 of them MMAs,
+// 2,900 arithmetic, 4,000 the operand writes into both CTAs and the fence behind them);
+// 44 with one lane of the MMA warp waiting by itself.
 #include "gelu.cuh"
 #include "mlp.cuh"
 #include "tc.cuh"
@@ -133,9 +134,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 ++it;
             }
         *issued = it;
-    } else if (warp == 1 && lane == 0) { // ---- MMA issuer, stores
+    } else if (warp == 1) { // ---- MMA issuer, stores: the warp waits as one, one lane issues
         bool ok = true, zload = false;
-        int it = 0;
+        int s = 0;
+        uint32_t round = 0;
+        const uint32_t lead = tc::elect_one(), d = __shfl_sync(0xffffffffu, tmem, 0);
         // phase p's results, complete in the operand tiles, to memory: each CTA its own
         // columns (the output gradient's 64 are one block: the first CTA)
         auto store = [&](int p) {
@@ -157,52 +160,62 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 }
                 tc::fence_after_sync();
                 if (p == 5) { // Z_2's tile has been read: Z_0 comes back into it
-                    tc::bulk_wait_all();
-                    tc::mbar_expect_tx(zbar, kZ);
-                    for (int kb = 0; kb < 2; ++kb)
-                        tc::tma_load_2d(zs + kb * kA, &maps.Z, zbar, (2 * (int)rank + kb) * BK, m0);
+                    if (lead) {
+                        tc::bulk_wait_all();
+                        tc::mbar_expect_tx(zbar, kZ);
+                        for (int kb = 0; kb < 2; ++kb)
+                            tc::tma_load_2d(zs + kb * kA, &maps.Z, zbar, (2 * (int)rank + kb) * BK, m0);
+                    }
                     zload = true;
                 }
             }
             const uint32_t idesc = p == 3 ? tc::idesc_bf16(BM, kOut / 2) : tc::idesc_bf16(BM, kHalf);
-            for (int kb = 0; kb < blocks_of(p); ++kb, ++it) {
-                const int s = it % kStages, r = it / kStages;
-                if (*abort_flag || !tc::mbar_wait(&full[s], r & 1, kWaitNs)) {
+            for (int kb = 0; kb < blocks_of(p); ++kb) {
+                if (!tc::mbar_wait(&full[s], round, kWaitNs)) {
                     ok = false;
                     break;
                 }
                 const uint32_t st = tc::smem_u32(smem + s * kStage);
                 const uint64_t a = tc::desc_sw128(p == 0 ? st : tc::smem_u32(hs + kb * kA));
                 const uint64_t w = tc::desc_sw128(st + kA);
+                if (lead) {
 #pragma unroll
-                for (int j = 0; j < BK / 16; ++j)
-                    tc::mma_bf16(tmem, a + 2 * j, w + 2 * j, idesc, (kb > 0 || j > 0) ? 1u : 0u);
-                tc::mma_commit(&empty[s]);
+                    for (int j = 0; j < BK / 16; ++j)
+                        tc::mma_bf16(d, a + 2 * j, w + 2 * j, idesc, (kb > 0 || j > 0) ? 1u : 0u);
+                    tc::mma_commit(&empty[s]);
+                }
+                if (++s == kStages) {
+                    s = 0;
+                    round ^= 1;
+                }
             }
             if (!ok) break;
-            tc::mma_commit_multicast(done, 3);
-            // the stores run beside the MMAs and the epilogues' arithmetic
-            if (p > 0) {
-                store(p - 1);
-                tc::bulk_wait_read_all();
+            if (lead) {
+                tc::mma_commit_multicast(done, 3);
+                // the stores run beside the MMAs and the epilogues' arithmetic
+                if (p > 0) {
+                    store(p - 1);
+                    tc::bulk_wait_read_all();
+                }
+                tc::mbar_arrive_cluster(tc::map_rank(tc::smem_u32(stored), 0));
+                tc::mbar_arrive_cluster(tc::map_rank(tc::smem_u32(stored), 1));
             }
-            tc::mbar_arrive_cluster(tc::map_rank(tc::smem_u32(stored), 0));
-            tc::mbar_arrive_cluster(tc::map_rank(tc::smem_u32(stored), 1));
+            __syncwarp();
         }
-        if (ok && tc::mbar_wait_cluster(ready, (kPhases - 1) & 1, kWaitNs)) {
-            store(kPhases - 1);
-        } else {
-            ok = false;
+        ok = ok && tc::mbar_wait_cluster(ready, (kPhases - 1) & 1, kWaitNs);
+        if (lead) {
+            if (ok) store(kPhases - 1);
+            tc::bulk_wait_all();
+            if (!ok) {
+                *abort_flag = 1;
+                atomicExch(c.err, PAAM_E_TIMEOUT);
+                if (zload) tc::mbar_wait(zbar, 0, kWaitNs / 4); // the copy has landed
+            }
+            // every MMA issued has completed before TMEM can be released
+            tc::mma_commit(fin);
+            tc::mbar_wait(fin, 0, kWaitNs);
         }
-        tc::bulk_wait_all();
-        if (!ok) {
-            *abort_flag = 1;
-            atomicExch(c.err, PAAM_E_TIMEOUT);
-            if (zload) tc::mbar_wait(zbar, 0, kWaitNs / 4); // the copy has landed
-        }
-        // every MMA this thread issued has completed before TMEM can be released
-        tc::mma_commit(fin);
-        tc::mbar_wait(fin, 0, kWaitNs);
+        __syncwarp();
     } else if (warp >= 2) { // ---- epilogues: one row per thread, 32 of the CTA's columns per warp
         const int q = warp & 3, cg = (warp - 2) >> 2; // TMEM lane quadrant, column group
         const int tr = 32 * q + lane;
