@@ -738,19 +738,7 @@ extern "C" int paam_rta_analyze_batch(paam_ctx *ctx, const paam_batch *b, const 
     }
     // launches of one graph run one after another; the first call's launches share its
     // scratch, so a graph that follows them on another stream waits for them
-    if (bm->first_open && stream != bm->first_stream) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(stream, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone) {
-            // a capture cannot wait for work outside it: the host does, once
-            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-            PAAM_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
-            const cudaError_t e = cudaEventSynchronize(bm->first_ev);
-            PAAM_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
-            PAAM_CUDA_TRY(e);
-        } else {
-            PAAM_CUDA_TRY(cudaStreamWaitEvent(stream, bm->first_ev, 0));
-        }
-    }
+    if (bm->first_open && stream != bm->first_stream) PAAM_CUDA_TRY(cudaStreamWaitEvent(stream, bm->first_ev, 0));
     bm->first_open = false;
     if (!same) {
         cudaStream_t cs = ctx->capture_stream;
