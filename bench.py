@@ -180,16 +180,18 @@ CONFIG_KERNEL = {0: "analyze_reg_kernel<8, 2>", 1: "analyze_fast_kernel<8, 16>",
 # instruction-issue side, against the issue peak of 152 SMs x 4 schedulers x 1
 # per clock.  Valid only while the kernels and the order they visit are
 # unchanged since the capture; a configuration without an entry reports null.
-# 26: analyze_lazy_kernel<16, 6> (1,022.1 MB), 28: analyze_lazy_kernel<16, 5> (959.0 MB);
-# neither defers a system of this workload, so configurations 24 and 23 run the
-# same kernels in the same order on it and take the same entries.
-_T26, _T28 = (949_534_464 + 72_603_904) / 500_000, (901_364_736 + 57_655_808) / 500_000
-TRAFFIC_PER_SYSTEM = {26: _T26, 24: _T26, 28: _T28, 23: _T28}
+# 26: analyze_lazy_kernel<16, 6> (1,031.6 MB), 28: analyze_lazy_kernel<16, 5> (954.1 MB),
+# 25: the same in index order (942.0 MB); none defers a system of this workload, so
+# configurations 24 and 23 run the same kernels in the same order as 26 and 28 on it
+# and take the same entries.
+_T26, _T28 = (948_914_176 + 82_642_688) / 500_000, (898_136_832 + 55_974_912) / 500_000
+_T25 = (887_197_184 + 54_826_240) / 500_000
+TRAFFIC_PER_SYSTEM = {26: _T26, 24: _T26, 28: _T28, 23: _T28, 25: _T25}
 # the same for the other workloads, keyed by (workload, launch configuration): the
 # uneven workload's step is the first pass, the 32-lane pass over the deferral list
 # and the 64-chain lazy kernel for the systems above 32 chains
-TRAFFIC_OTHER = {("cfg3", 26): (867_346_688 + 40_391_936 + 346_479_616 + 16_131_584 + 109_261_824 + 1_899_520) / 500_000,
-                 ("cfg3", 28): (849_617_152 + 30_518_528 + 346_491_904 + 16_272_896 + 109_204_480 + 1_914_624) / 500_000}
+TRAFFIC_OTHER = {("cfg3", 26): (867_767_552 + 45_668_352 + 346_492_672 + 20_750_336 + 109_225_728 + 4_857_856) / 500_000,
+                 ("cfg3", 28): (848_869_632 + 31_267_072 + 346_433_280 + 20_746_240 + 109_206_272 + 4_874_496) / 500_000}
 
 
 def traffic_per_system(workload: str, cfg_index: int):
@@ -198,8 +200,8 @@ def traffic_per_system(workload: str, cfg_index: int):
     return TRAFFIC_OTHER.get((workload, cfg_index))
 
 
-WARP_INST_PER_SYSTEM = {26: 551_079_382 / 500_000, 24: 551_079_382 / 500_000, 28: 531_338_213 / 500_000,
-                        23: 531_338_213 / 500_000}
+WARP_INST_PER_SYSTEM = {26: 481_186_547 / 500_000, 24: 481_186_547 / 500_000, 28: 457_257_799 / 500_000,
+                        23: 457_257_799 / 500_000, 25: 458_244_913 / 500_000}
 ISSUE_PEAK = 152 * 4 * 2.07e9  # warp-instructions / s at the 2070 MHz maximum SM clock
 
 

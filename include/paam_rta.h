@@ -79,8 +79,8 @@ typedef struct paam_model paam_model;
  *                  0).  Each accelerator has its own server (rule R1) and is
  *                  analysed on its own: buckets, same-bucket blocking and hps
  *                  are per accelerator, and H_c sums the per-accelerator
- *                  handling times.  A batch that uses a second accelerator
- *                  is analysed by the exact int64 kernel (slower)
+ *                  handling times.  Systems outside the 32-bit bound take the
+ *                  exact int64 kernel (slower)
  *   exec_core[x]   CPU core of executor x, >= 0
  *   exec_prio[x]   executor (process) priority, larger = higher, distinct among
  *                  executors of one core; NULL = derived as the highest chain
@@ -123,8 +123,7 @@ typedef struct {
  *                  callback i's segments of (Lemma 2 bound + eps) of a
  *                  lower-priority chain on the executor, and a segment
  *                  without a bound (above its chain's deadline) makes the
- *                  chain PAAM_ST_OVERRUN.  Mode 1 runs the exact int64 kernel
- *                  for every system (slower).  Other values: PAAM_E_INVAL
+ *                  chain PAAM_ST_OVERRUN.  Other values: PAAM_E_INVAL
  *   eps_ns         per-request server overhead epsilon (Eq. 1), 0..2^32
  *   kappa_ns       device preemption cost kappa, A* = A + 2 kappa, 0..2^32
  */
@@ -294,12 +293,14 @@ int paam_rta_analyze_host(paam_ctx *ctx, const paam_systems_view *v, const paam_
  *                          a row is a candidate row of
  *                          paam_rta_search_priorities.
  *
- * Every trial of every system at one level is analysed in one launch of the
- * exact int64 kernel, which stops each trial once chain c is done.  Scratch
- * is taken from the stream's pool (at most about 512 MB; larger batches run
- * in system chunks).  The call synchronises `stream`.  Errors: PAAM_E_INVAL
- * (bad sizes or options), PAAM_E_RANGE (eps/kappa above the cap),
- * PAAM_E_STATE (a batch of another context), PAAM_E_NOMEM, PAAM_E_CUDA.
+ * A batch with one accelerator, under the literal reading, runs the levels of
+ * each system of up to 32 chains inside the 32-bit bound in one kernel; for the
+ * others all trials of one level are analysed in one launch of the exact int64
+ * kernel.  Scratch is taken from the stream's pool (at most about 512 MB;
+ * larger batches run in system chunks).  The call synchronises `stream`.
+ * Errors: PAAM_E_INVAL (bad sizes or options), PAAM_E_RANGE (eps/kappa above
+ * the cap), PAAM_E_STATE (a batch of another context), PAAM_E_NOMEM,
+ * PAAM_E_CUDA.
  */
 int paam_rta_audsley_order(paam_ctx *ctx, const paam_batch *batch, const paam_analysis_opts *opts, int32_t nmax,
                            int16_t *ranks_out, void *stream);

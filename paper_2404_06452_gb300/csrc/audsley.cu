@@ -36,7 +36,7 @@ using namespace paam_cand;
 // With many systems the trials themselves are the limit (issue, 58% of the slots,
 // and the last systems' levels): one group per system.  A batch too small to fill
 // the chip is bound by one system's chain of levels: two groups, or a whole block
-// of 16 (LG = 16) or 8 (LG = 32).  10,000 systems of 16 chains: 0.41 ms, where the
+// of 16 (LG = 16) or 8 (LG = 32).  10,000 systems of 16 chains: 0.37 ms, where the
 // launches per level took 3.8 ms (trial rows 0.6, trials 3.0, picks 0.15).
 template <int LG, int GPS>
 __global__ void __launch_bounds__(256, LG == 16 ? 4 : 3)
