@@ -577,9 +577,14 @@ const LaunchCfg kLaunchCfgs[] = {
 const int kNumLaunchCfgs = (int)(sizeof(kLaunchCfgs) / sizeof(kLaunchCfgs[0]));
 static_assert(kDefaultLaunchCfg < (int)(sizeof(kLaunchCfgs) / sizeof(kLaunchCfgs[0])), "default configuration");
 
-int paam_enqueue_analysis(const paam_batch *b, const AnalysisParams &p, const LaunchCfg &cfg, int64_t *R,
+int paam_enqueue_analysis(const paam_batch *b, const AnalysisParams &opts, const LaunchCfg &cfg, int64_t *R,
                           uint8_t *status, uint8_t *verdict, cudaStream_t stream, int *n_kernels)
 {
+    // floor(rank n / |U|) (R2) puts the same users together for every n >= |U|: each has a
+    // bucket of its own.  No system has more users than chains, so the kernels see at most
+    // PAAM_MAX_CHAINS buckets and their 32-bit products of rank and buckets are exact.
+    AnalysisParams p = opts;
+    if (p.n_buckets > PAAM_MAX_CHAINS) p.n_buckets = PAAM_MAX_CHAINS;
     LaunchFn small = find_variant(cfg.impl_small, cfg.g_small, cfg.maxn_small);
     LaunchFn bigfn = cfg.impl_big == kImplBigLazy32 ? launch_reg<32, 2> : find_variant(cfg.impl_big, cfg.g_big, 64);
     if (!small || !bigfn) return PAAM_E_INVAL;
