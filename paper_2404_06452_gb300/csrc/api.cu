@@ -141,6 +141,7 @@ __device__ __noinline__ bool range_exact(const BatchDev &b, int64_t c0, int64_t 
         Cmax = fmax(Cmax, Ec + fmax(D, dc * OV) + Sc);
         Base = fmax(Base, Ec + Sc + dc * OV);
         dseg_max = fmax(dseg_max, dc);
+        if (Cmax >= 2.305843009213694e18) return false; // past the bound below by itself
     }
     // the largest value an iterate can take: interference over n chains with at most
     // ceil(Dmax/Tmin)+1 arrivals each, plus blocking and the chain's own demand
@@ -364,7 +365,7 @@ __global__ void __launch_bounds__(kValThreads, kValBlocks) validate_kernel(const
         const uint32_t S = __reduce_add_sync(gm, as < kLaneCap ? (uint32_t)as : kLaneCap);
         const float M = (float)__reduce_max_sync(gm, amax) + 0x1p33f;
         const bool large = __any_sync(gm, es >= kLaneCap || as >= kLaneCap || thi != 0) || E >= kSumCap ||
-                           S >= kSumCap || dl >= (1 << 20);
+                           S >= kSumCap || dl >= (1 << 20) || b1 - b0 >= (1 << 20); // longer sums may have wrapped
         const float ratio = Dm / Tm, nf = (float)n, d32 = (float)dl * 0x1p32f;
         const float C = (float)E + fmaxf(Dm, d32) + (float)S + 2.0f * d32;
         if (large || !((nf * (ratio + 2.0f) + 3.0f) * C + (float)dl * M < 0x1p60f &&
