@@ -186,7 +186,8 @@ void paam_batch_free(paam_batch *b);
  * launch configuration.  The first call for a given (outputs, options,
  * launch configuration) launches the analysis; the second captures it into a
  * CUDA graph owned by the batch, and later calls with the same key replay it
- * on `stream`.  A batch may be
+ * on `stream`.  Analyses of one batch run one after another in the order of
+ * their calls, on whatever streams: they share its scratch.  A batch may be
  * analysed by one host thread at a time.  Errors: PAAM_E_INVAL (NULL outputs, n_buckets < 1),
  * PAAM_E_RANGE (eps or kappa above PAAM_MAX_OVERHEAD), PAAM_E_INVAL
  * (blocking_mode not 0 or 1), PAAM_E_CUDA (launch failure).

@@ -545,7 +545,7 @@ extern "C" void paam_batch_free(paam_batch *b)
     if (!b) return;
     cudaSetDevice(b->ctx->device);
     if (b->graph) cudaGraphExecDestroy(b->graph);
-    if (b->first_ev) cudaEventDestroy(b->first_ev);
+    if (b->last_ev) cudaEventDestroy(b->last_ev);
     if (b->block) cudaFree(b->block);
     free(b);
 }
@@ -688,6 +688,13 @@ static AnalysisParams params_of(const paam_analysis_opts *o)
     return p;
 }
 
+// Work enqueued on `stream` after this runs after the batch's last analysis.
+static int follow_last_analysis(const paam_batch *b, cudaStream_t stream)
+{
+    if (b->used) PAAM_CUDA_TRY(cudaStreamWaitEvent(stream, b->last_ev, 0));
+    return PAAM_OK;
+}
+
 extern "C" int paam_rta_analyze_batch(paam_ctx *ctx, const paam_batch *b, const paam_analysis_opts *o,
                                       int64_t *R, uint8_t *status, uint8_t *verdict, void *stream_)
 {
@@ -711,12 +718,14 @@ extern "C" int paam_rta_analyze_batch(paam_ctx *ctx, const paam_batch *b, const 
             cudaGraphExecDestroy(bm->graph);
             bm->graph = nullptr;
         }
+        bm->apart = true;
         bm->graph_key.R = R;
         bm->graph_key.status = status;
         bm->graph_key.verdict = verdict;
         bm->graph_key.p = p;
         bm->graph_key.cfg_index = bm->cfg_index;
     };
+    if (!bm->last_ev) PAAM_CUDA_TRY(cudaEventCreateWithFlags(&bm->last_ev, cudaEventDisableTiming));
     if (!same && !(bm->key_seen && key_same)) {
         bm->key_seen = true;
         set_key();
@@ -725,22 +734,16 @@ extern "C" int paam_rta_analyze_batch(paam_ctx *ctx, const paam_batch *b, const 
             // the first call with these outputs, options and configuration: launched as it
             // is (a graph's capture and instantiation cost more than they save one call;
             // load + analysis + free of 200,000 systems 709 -> 643 us)
-            if (!bm->first_ev) PAAM_CUDA_TRY(cudaEventCreateWithFlags(&bm->first_ev, cudaEventDisableTiming));
+            if (follow_last_analysis(b, stream) != PAAM_OK) return PAAM_E_CUDA;
             int nk = 0;
             rc = paam_enqueue_analysis(b, p, kLaunchCfgs[bm->cfg_index], R, status, verdict, stream, &nk);
-            if (rc != PAAM_OK) return rc;
-            paam_count_launch((unsigned)nk);
-            PAAM_CUDA_TRY(cudaEventRecord(bm->first_ev, stream));
-            bm->first_stream = stream;
-            bm->first_open = true;
-            return PAAM_OK;
+            if (cudaEventRecord(bm->last_ev, stream) != cudaSuccess && rc == PAAM_OK) rc = PAAM_E_CUDA;
+            bm->used = true;
+            if (rc == PAAM_OK) paam_count_launch((unsigned)nk);
+            return rc;
         }
         cudaGetLastError();
     }
-    // launches of one graph run one after another; the first call's launches share its
-    // scratch, so a graph that follows them on another stream waits for them
-    if (bm->first_open && stream != bm->first_stream) PAAM_CUDA_TRY(cudaStreamWaitEvent(stream, bm->first_ev, 0));
-    bm->first_open = false;
     if (!same) {
         cudaStream_t cs = ctx->capture_stream;
         PAAM_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
@@ -761,7 +764,12 @@ extern "C" int paam_rta_analyze_batch(paam_ctx *ctx, const paam_batch *b, const 
         }
         bm->graph_kernels = nk;
     }
+    // launches of one graph follow one another on any streams
+    if (bm->apart && follow_last_analysis(b, stream) != PAAM_OK) return PAAM_E_CUDA;
     PAAM_CUDA_TRY(cudaGraphLaunch(bm->graph, stream));
+    PAAM_CUDA_TRY(cudaEventRecord(bm->last_ev, stream));
+    bm->used = true;
+    bm->apart = false;
     paam_count_launch((unsigned)bm->graph_kernels);
     return PAAM_OK;
 }
@@ -788,6 +796,8 @@ extern "C" int paam_rta_autotune(paam_ctx *ctx, paam_batch *b, const paam_analys
     PAAM_CUDA_TRY(cudaSetDevice(ctx->device));
     cudaStream_t stream = (cudaStream_t)stream_;
     const AnalysisParams p = params_of(o);
+    rc = follow_last_analysis(b, stream);
+    if (rc != PAAM_OK) return rc;
     void *tmp = nullptr;
     const size_t rb = 8 * (size_t)b->n_chain, sb = (size_t)b->n_chain, vb = (size_t)b->n_sys;
     if (cudaMallocAsync(&tmp, rb + sb + vb + 64, stream) != cudaSuccess) {

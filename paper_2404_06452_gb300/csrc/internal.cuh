@@ -192,9 +192,12 @@ struct paam_batch {
     // the analysis captured as a CUDA graph at the second call with one key, replayed
     // while the key matches (key_seen: the key holds some earlier call's values)
     cudaGraphExec_t graph;
-    bool key_seen, first_open; // first_open: the first call's launches may still run
-    cudaEvent_t first_ev;      // recorded after them on first_stream
-    cudaStream_t first_stream;
+    bool key_seen;
+    // the batch's lists and counters serve one analysis at a time, on whatever streams:
+    // last_ev is recorded after each one (used: it has been); apart: the last one was not
+    // a launch of the present graph
+    bool used, apart;
+    cudaEvent_t last_ev;
     int graph_kernels;
     struct {
         int64_t *R;
