@@ -190,7 +190,8 @@ void paam_batch_free(paam_batch *b);
  * their calls, on whatever streams: they share its scratch.  A batch may be
  * analysed by one host thread at a time.  Errors: PAAM_E_INVAL (NULL outputs, n_buckets < 1),
  * PAAM_E_RANGE (eps or kappa above PAAM_MAX_OVERHEAD), PAAM_E_INVAL
- * (blocking_mode not 0 or 1), PAAM_E_CUDA (launch failure).
+ * (blocking_mode not 0 or 1), PAAM_E_CUDA (launch failure; also a stream that
+ * is being captured, of which nothing is touched: the capture stays valid).
  */
 int paam_rta_analyze_batch(paam_ctx *ctx, const paam_batch *batch, const paam_analysis_opts *opts,
                            int64_t *R, uint8_t *status, uint8_t *verdict, void *stream);

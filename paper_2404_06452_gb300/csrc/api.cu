@@ -706,6 +706,13 @@ extern "C" int paam_rta_analyze_batch(paam_ctx *ctx, const paam_batch *b, const 
     if (b->n_sys == 0) return PAAM_OK;
     PAAM_CUDA_TRY(cudaSetDevice(ctx->device));
     cudaStream_t stream = (cudaStream_t)stream_;
+    // a graph cannot be launched into a capture, nor can a capture wait for the batch's last
+    // analysis: refused before the capture is touched
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return PAAM_E_CUDA;
+    }
     const AnalysisParams p = params_of(o);
     paam_batch *bm = const_cast<paam_batch *>(b); // the captured graph is a cache inside the handle
     const bool key_same = bm->graph_key.R == R && bm->graph_key.status == status &&
@@ -729,20 +736,16 @@ extern "C" int paam_rta_analyze_batch(paam_ctx *ctx, const paam_batch *b, const 
     if (!same && !(bm->key_seen && key_same)) {
         bm->key_seen = true;
         set_key();
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
-            // the first call with these outputs, options and configuration: launched as it
-            // is (a graph's capture and instantiation cost more than they save one call;
-            // load + analysis + free of 200,000 systems 709 -> 643 us)
-            if (follow_last_analysis(b, stream) != PAAM_OK) return PAAM_E_CUDA;
-            int nk = 0;
-            rc = paam_enqueue_analysis(b, p, kLaunchCfgs[bm->cfg_index], R, status, verdict, stream, &nk);
-            if (cudaEventRecord(bm->last_ev, stream) != cudaSuccess && rc == PAAM_OK) rc = PAAM_E_CUDA;
-            bm->used = true;
-            if (rc == PAAM_OK) paam_count_launch((unsigned)nk);
-            return rc;
-        }
-        cudaGetLastError();
+        // the first call with these outputs, options and configuration: launched as it is (a
+        // graph's capture and instantiation cost more than they save one call; load +
+        // analysis + free of 200,000 systems 709 -> 643 us)
+        if (follow_last_analysis(b, stream) != PAAM_OK) return PAAM_E_CUDA;
+        int nk = 0;
+        rc = paam_enqueue_analysis(b, p, kLaunchCfgs[bm->cfg_index], R, status, verdict, stream, &nk);
+        if (cudaEventRecord(bm->last_ev, stream) != cudaSuccess && rc == PAAM_OK) rc = PAAM_E_CUDA;
+        bm->used = true;
+        if (rc == PAAM_OK) paam_count_launch((unsigned)nk);
+        return rc;
     }
     if (!same) {
         cudaStream_t cs = ctx->capture_stream;
