@@ -215,9 +215,13 @@ __device__ __forceinline__ void range_per_chain(const ValidateArgs &a, int64_t s
 // Every system of a batch that validate_kernel found valid but could not place
 // clearly inside the limits (rare: periods of seconds, thousands of segments,
 // magnitudes near the limits); a launch of its own, so that the pass that every
-// batch takes keeps its registers.
+// batch takes keeps its registers.  A block returns at once where that pass left nothing
+// open or found the batch invalid (one thread's reading, for all: other blocks may refuse
+// a system meanwhile).
 __global__ void __launch_bounds__(kValThreads) range_kernel(const __grid_constant__ ValidateArgs a)
 {
+    const volatile int32_t *err = a.err;
+    if (__syncthreads_or(threadIdx.x == 0 && (err[0] != 0 || err[1] == 0))) return;
     const int lane = threadIdx.x % G;
     const unsigned gm = ((1u << G) - 1u) << (threadIdx.x & 31u & ~(unsigned)(G - 1));
     const int64_t stride = (int64_t)gridDim.x * (kValThreads / G);

@@ -340,9 +340,10 @@ constexpr uint32_t kIterCap = (uint32_t)PAAM_MAX_ITER;
 int paam_enqueue_analysis(const paam_batch *b, const AnalysisParams &p, const LaunchCfg &cfg, int64_t *R,
                           uint8_t *status, uint8_t *verdict, cudaStream_t stream, int *n_kernels);
 
-// Validation kernel (api.cu): err and stats as in ValidateWords.  Once the
-// words are on the host and paam_validate_undecided says so, the batch (valid so
-// far) also takes paam_launch_validate_rest, which adds to the same words.  The
+// Validation kernel (api.cu): err and stats as in ValidateWords.  A batch with
+// systems that it leaves open (paam_validate_undecided on the words, once they are on
+// the host) also takes paam_launch_validate_rest, which adds to the same words and
+// returns at once where nothing is open: it may be enqueued unasked.  The
 // maxima of a chain's E, A and segments may be their system's sums (below 2^29),
 // which only ever sends a batch to one kernel more.
 int paam_launch_validate(const paam_batch *b, const int32_t *acc, int32_t *err, unsigned long long *stats,
