@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(kGemmThreads, 2) tc_gemm_kernel(const __grid_c
         const int half = (warp - 2) >> 2;
         const int row = m0 + 32 * q + lane;
         bool ok = nkb > 0;
-        if (ok && !tc::mbar_wait(done, 0, kWaitNs)) {
+        if (ok && !tc::warp_ok(tc::mbar_wait(done, 0, kWaitNs))) {
             ok = false;
             *abort_flag = 1;
             atomicExch(err, PAAM_E_TIMEOUT);
@@ -412,7 +412,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
         int i = 0;
         for (int tile = blockIdx.x; tile < m_tiles; tile += gridDim.x, ++i) {
             const int b = i & 1;
-            if (*abort_flag || !tc::mbar_wait(&acc_full[b], (i >> 1) & 1, kWaitNs)) {
+            if (!tc::warp_ok(!*abort_flag && tc::mbar_wait(&acc_full[b], (i >> 1) & 1, kWaitNs))) {
                 *abort_flag = 1;
                 atomicExch(err, PAAM_E_TIMEOUT);
                 break;

@@ -147,6 +147,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t a0 = tc::smem_u32(smem), w0 = tc::smem_u32(ring);
         const uint32_t d0 = __shfl_sync(0xffffffffu, tmem, 0);
         const bool ok = walk(m_tiles, [&](int l, int t, int u) {
+            // no vote here: the warp executes nothing together before the __syncwarp at the
+            // end, where a lane that gives up waits for the others
             if (*abort_flag) return false;
             if (l > 0 ? !tc::mbar_wait(&ready[t], (3 * u + l - 1) & 1, kWaitNs)
                       : (u > 0 && !tc::mbar_wait(&out_read[t], (u - 1) & 1, kWaitNs)))
@@ -209,7 +211,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int i = 0; i < 6; ++i) {
                 const int l = i >> 1, t = i & 1;
                 if (tile_of(u, t) >= m_tiles) continue;
-                if (*abort_flag || !tc::mbar_wait(&acc[t], (3 * u + l) & 1, kWaitNs)) {
+                if (!tc::warp_ok(!*abort_flag && tc::mbar_wait(&acc[t], (3 * u + l) & 1, kWaitNs))) {
                     give_up();
                     ok = false;
                     break;
@@ -263,7 +265,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int64_t sys = c.sys_list ? (int64_t)c.sys_list[at] : at;
                     n = (int)(c.sys_off[sys + 1] - c.sys_off[sys]);
                 }
-                if (*abort_flag || !tc::mbar_wait(&acc_out[t], u & 1, kWaitNs)) {
+                if (!tc::warp_ok(!*abort_flag && tc::mbar_wait(&acc_out[t], u & 1, kWaitNs))) {
                     give_up();
                     ok = false;
                     break;

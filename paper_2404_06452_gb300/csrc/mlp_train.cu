@@ -154,7 +154,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         };
         for (int p = 0; p < kPhases && ok; ++p) {
             if (p > 0) {
-                if (*abort_flag || !tc::mbar_wait_cluster(ready, (p - 1) & 1, kWaitNs)) {
+                if (!tc::warp_ok(!*abort_flag && tc::mbar_wait_cluster(ready, (p - 1) & 1, kWaitNs))) {
                     ok = false;
                     break;
                 }
@@ -171,10 +171,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             }
             const uint32_t idesc = p == 3 ? tc::idesc_bf16(BM, kOut / 2) : tc::idesc_bf16(BM, kHalf);
             for (int kb = 0; kb < blocks_of(p); ++kb) {
-                if (!tc::mbar_wait(&full[s], round, kWaitNs)) {
-                    ok = false;
-                    break;
-                }
+                ok = tc::mbar_wait(&full[s], round, kWaitNs);
+                if (!ok) break; // to the vote below
                 const uint32_t st = tc::smem_u32(smem + s * kStage);
                 const uint64_t a = tc::desc_sw128(p == 0 ? st : tc::smem_u32(hs + kb * kA));
                 const uint64_t w = tc::desc_sw128(st + kA);
@@ -189,6 +187,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     round ^= 1;
                 }
             }
+            ok = tc::warp_ok(ok);
             if (!ok) break;
             if (lead) {
                 tc::mma_commit_multicast(done, 3);
@@ -202,7 +201,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             }
             __syncwarp();
         }
-        ok = ok && tc::mbar_wait_cluster(ready, (kPhases - 1) & 1, kWaitNs);
+        ok = ok && tc::warp_ok(tc::mbar_wait_cluster(ready, (kPhases - 1) & 1, kWaitNs));
         if (lead) {
             if (ok) store(kPhases - 1);
             tc::bulk_wait_all();
@@ -224,8 +223,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const uint32_t ready_peer = tc::map_rank(tc::smem_u32(ready), rank ^ 1);
 #pragma unroll 1
         for (int p = 0; p < kPhases; ++p) {
-            if (*abort_flag || !tc::mbar_wait_cluster(done, p & 1, kWaitNs) ||
-                (p == 6 && !tc::mbar_wait(zbar, 0, kWaitNs))) {
+            if (!tc::warp_ok(!*abort_flag && tc::mbar_wait_cluster(done, p & 1, kWaitNs) &&
+                             (p < 6 || tc::mbar_wait(zbar, 0, kWaitNs)))) {
                 *abort_flag = 1;
                 atomicExch(c.err, PAAM_E_TIMEOUT);
                 break;
@@ -295,8 +294,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                                                        __uint_as_float(v[2 * i + 1]) * gelu_grad(zf.y));
                     }
                 }
-                if (!tc::mbar_wait_cluster(stored, p & 1, kWaitNs)) {
-                    *abort_flag = 1; // every lane gives up: the warp leaves at its next phase
+                if (!tc::warp_ok(tc::mbar_wait_cluster(stored, p & 1, kWaitNs))) {
+                    *abort_flag = 1; // the warp leaves at its next phase
                     atomicExch(c.err, PAAM_E_TIMEOUT);
                 }
                 const uint4 *o4 = reinterpret_cast<const uint4 *>(out);

@@ -65,6 +65,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64
     return true;
 }
 
+// For a warp that waits as one: `ok` of every lane, the same in all of them.  Each lane's
+// wait runs out by its own clock, and a lane that gave up alone would leave the others in
+// instructions the whole warp must execute together (tcgen05.ld, shuffles), with no limit.
+__device__ __forceinline__ bool warp_ok(bool ok) { return __all_sync(0xffffffffu, ok); }
+
 // true in one lane of the (whole) warp
 __device__ __forceinline__ uint32_t elect_one()
 {
