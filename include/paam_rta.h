@@ -457,8 +457,8 @@ int paam_measure_preemption(int device, int kind, int iters, float *delay_us, fl
  * configurations (lanes per system, chain-table size of the first pass, lanes
  * per system for systems with more chains, CTA size, static shares or a
  * device work queue, index or size order of the systems); every one produces
- * bit-identical results.  A batch starts with configuration 12 (16 lanes per
- * system, work queue).
+ * bit-identical results.  A batch starts with configuration 28 (16 lanes per
+ * system, then a warp per larger system; work queue, size order).
  *
  * paam_rta_autotune times every configuration on the batch itself (the
  * analysis is run 6 times per configuration, the first run discarded, and
@@ -505,8 +505,9 @@ int paam_rta_get_launch_config(const paam_batch *batch);
  *   - n_sys above PAAM_NOALLOC_MAX_SYS is rejected with PAAM_E_RANGE (split
  *     larger batches into several calls);
  *   - the input is validated exactly as paam_rta_load_systems does, so the
- *     call synchronises `stream` once (after validation) and returns the
- *     same error codes; the analysis itself is then enqueued on `stream`;
+ *     call synchronises `stream` after validation (twice where systems need
+ *     its second pass) and returns the same error codes; the analysis itself
+ *     is then enqueued on `stream`;
  *   - every call looks up the array's device address on the current device
  *     (a lookup, no allocation), so the address stays right across a
  *     cudaDeviceReset; the first call on a device also reads two device

@@ -23,7 +23,7 @@
 // narrow one, go to b.list_big (the 32-lane pass of this kernel over that list,
 // then analyze_lazy64.cu for those above 32 chains); systems outside the 32-bit
 // bound to b.list_wide (the int64 kernel).  One accelerator: Lemma 4 as printed
-// (blocking_mode 0) in analysis, candidate and target mode, and the safe reading
+// (blocking_mode 0) in analysis and candidate mode, and the safe reading
 // (blocking_mode 1, 16 lanes); several accelerators keep their kernel
 // (analyze_lazy_acc.cu), and the larger systems of both options theirs
 // (analyze_lazy_big.cu).

@@ -827,7 +827,13 @@ __device__ void big_system(const BatchDev &b, const AnalysisParams &p, int64_t i
     if (lane == 0 && verdict) verdict[sys] = sched == all ? 1 : 0;
 }
 
-constexpr int kWarps = 4; // systems per block: 45 KB of tables at most
+constexpr int kWarps = 4; // systems per block
+// The block's tables: 63.5 KB with four accelerators and 51.2 KB under the safe reading
+// (up to 64 chains), above the 48 KB that need no attribute.
+constexpr size_t kBigTables = 64 << 10;
+static_assert(sizeof(BigSmem<2, PAAM_MAX_ACC, false>) * kWarps <= kBigTables &&
+                  sizeof(BigSmem<2, 1, true>) * kWarps <= kBigTables,
+              "the largest tables of a block");
 
 template <int CPL, int NACC, bool SAFE>
 __global__ void __launch_bounds__(32 * kWarps) analyze_lazy_big_kernel(const __grid_constant__ BatchDev b,

@@ -95,8 +95,8 @@ extern "C" void paam_destroy(paam_ctx *c)
 // precision (16 cycles per warp instruction on this chip).  A thread per system,
 // sums in double precision: 740 us for 200,000 systems of 8-16 chains, 7,290 us for
 // 1,000,000 of 2-64, 28 us for 1,000 of 4; now 140, 870 and 17 us (16 lanes per
-// system: 202 and 1,002 us; 8 lanes: 158 and 940; six or eight blocks per SM spill:
-// 154 us).  The one read of every table would take 55 us for the 200,000.
+// system: 202 and 1,002 us; 8 lanes: 158 and 940).  Five blocks per SM (48 registers, 104
+// bytes of spill stores) beat six and eight, which spill more, 154 us.  The one read of every table would take 55 us for the 200,000.
 // ---------------------------------------------------------------------------
 
 constexpr int G = 4, kValThreads = 256, kValBlocks = 5;

@@ -43,10 +43,12 @@ size_t n_params()
 }
 
 // ---- labels: clip(R / D, 0, 2) for schedulable chains, 2 otherwise, -1 for padding.
-// R / D rounded once to single precision, without double precision (whose divide
-// alone bound this kernel: 72 us for 100,000 systems, 39 us now): with q near 2^24 R / D
-// the remainder 2^24 R - q D is exact in 64 bits for R < 2^38, and q plus the
-// remainder over D, both small floats, is added once.  Four slots per thread.
+// R / D in single precision without double precision (whose divide alone bound this
+// kernel: 72 us for 100,000 systems, 39 us now): with q near 2^24 R / D the remainder
+// 2^24 R - q D is exact in 64 bits for R < 2^38, and q plus the remainder over D, both
+// small floats, is added once: rounded correctly but within some 2^-22 of a tie (2 of 20
+// million random quotients differ, in the last bit, from the double one's rounding).
+// Four slots per thread.
 __device__ __forceinline__ float ratio_of(int64_t R, int64_t D)
 {
     if (R >> 38 || D >> 38) return (float)((double)R / (double)D);
